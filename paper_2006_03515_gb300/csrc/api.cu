@@ -56,14 +56,24 @@ static void free_plan(Plan* p) {
     dev_free(p->vtab);
     for (auto& o : p->ops)
         for (DevBuf* b : {&o.G1, &o.Vb, &o.Ub, &o.Vt, &o.T, &o.Mc, &o.Lo, &o.T32, &o.Ub32, &o.Vb32, &o.Vt32, &o.Lo32, &o.Mc32, &o.ozG1, &o.ozEr,
-                          &o.Thi, &o.Tlo, &o.Lhi, &o.Llo, &o.Mhi, &o.Mlo})
+                          &o.Ttc, &o.Ltc, &o.Mtc})
             dev_free(*b);
     for (DevBuf* b : {&p->surf, &p->ctab, &p->ctab32, &p->cheb_A, &p->pts, &p->loc32, &p->w, &p->sigma, &p->leaf_of, &p->leaves, &p->p2m_boxes,
-                      &p->q, &p->Isort, &p->chk, &p->chkx, &p->cu, &p->cu32, &p->chi, &p->clo, &p->cexp, &p->ozBox, &p->ozEb, &p->dd, &p->phid, &p->phiu,
+                      &p->q, &p->Isort, &p->chk, &p->chkx, &p->cu, &p->cu32, &p->chl, &p->cexp, &p->ozBox, &p->ozEb, &p->dd, &p->phid, &p->phiu,
                       &p->far, &p->wleaves, &p->host_I, &p->host_S, &p->err,
-                      &p->tc_tiles, &p->tc_boxes, &p->tc_slots, &p->ptab, &p->l2l_slots, &p->m2m_tiles, &p->m2m_slots, &p->stage32, &p->m2m_hi, &p->m2m_lo, &p->apply_part, &p->nf_utab, &p->nf_Thi, &p->nf_Tlo, &p->nf_tiles,
-                      &p->nf_slots, &p->nf_boxes, &p->nf_qhi, &p->nf_qlo, &p->nf_qexp, &p->nf_near, &p->lat_P, &p->lat_Q, &p->lat_Thi, &p->lat_Tlo, &p->lat_iota, &p->lat_slots, &p->lat_fst, &p->lat_Mimg, &p->lat_Mer, &p->nf_ref})
+                      &p->tc_tiles, &p->tc_boxes, &p->tc_slots, &p->ptab, &p->l2l_slots, &p->m2m_tiles, &p->m2m_slots, &p->stage32, &p->m2m_chl, &p->apply_part, &p->nf_utab, &p->nf_Ttc, &p->nf_tiles,
+                      &p->nf_slots, &p->nf_boxes, &p->nf_qhl, &p->nf_qexp, &p->nf_near, &p->lat_P, &p->lat_Q, &p->lat_Ttc, &p->lat_iota, &p->lat_slots, &p->lat_fst, &p->lat_Mimg, &p->lat_Mer, &p->nf_ref})
         dev_free(*b);
+    auto free_sched = [](TcSched& s) {
+        for (DevBuf* b : {&s.pre, &s.first, &s.src, &s.meta, &s.part}) dev_free(*b);
+    };
+    free_sched(p->sch_m2l);
+    free_sched(p->sch_near);
+    free_sched(p->sch_lat);
+    for (int l = 0; l <= kMaxLevel; ++l) {
+        free_sched(p->sch_l2l[l]);
+        free_sched(p->sch_m2m[l]);
+    }
     for (auto& L : p->lv) {
         for (DevBuf* b : {&L.all, &L.leafs, &L.nonleaf, &L.m2l_tiles, &L.m2l_slots, &L.m2l_slot_off, &L.xboxes,
                           &L.m2l_slots128, &L.m2l_boxes, &L.parents, &L.par_kids, &L.upb,

@@ -408,6 +408,8 @@ int build_eval_data(Plan& p) {
         p.tc_ntiles = (int)tiles.size();
         if (!tiles.empty())
             KF_CUDA(cudaMemcpyAsync(p.tc_tiles.p, tiles.data(), tiles.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
+        KF_TRY(tc_sched_build(st, ptr<int4>(p.tc_tiles), ptr<int32_t>(p.tc_boxes), ptr<int32_t>(p.vtab), kOffsetSlots,
+                              ptr<int32_t>(p.tc_slots), p.tc_ntiles, p.R, p.num_sms, p.sch_m2l));
         // L2L through the same kernel: per child tile the parent at its octant's slot, the
         // parent level's L2L matrices as FP16 hi / lo tables (KIFMM_L2L=simt keeps the SIMT apply)
         const char* l2l = std::getenv("KIFMM_L2L");
@@ -425,10 +427,14 @@ int build_eval_data(Plan& p) {
             KF_LAUNCH();
             for (int l = 2; l + 1 < t.nlevels; ++l) {
                 LevelOps& op = p.ops[l];
-                KF_TRY(dev_alloc(op.Lhi, (size_t)m2l_tc_table_elems(p.R, 8) * 2));
-                KF_TRY(dev_alloc(op.Llo, (size_t)m2l_tc_table_elems(p.R, 8) * 2));
-                KF_TRY(m2l_tc_prepare(st, ptr<double>(op.Lo), p.R, op.Lhi.p, op.Llo.p, &op.l2l_sT, 8));
+                KF_TRY(dev_alloc(op.Ltc, (size_t)m2l_tc_table_elems(p.R, 8) * 2));
+                KF_TRY(m2l_tc_prepare(st, ptr<double>(op.Lo), p.R, op.Ltc.p, &op.l2l_sT, 8));
             }
+            for (int l = 3; l < t.nlevels; ++l)
+                KF_TRY(tc_sched_build(st, ptr<int4>(p.tc_tiles) + p.tc_first[l], ptr<int32_t>(p.tc_boxes),
+                                      ptr<int32_t>(p.ptab), 8,
+                                      ptr<int32_t>(p.l2l_slots) + (int64_t)p.tc_first[l] * kSlotStride, p.tc_count[l],
+                                      p.R, p.num_sms, p.sch_l2l[l]));
         }
         // M2M translations likewise: per parent tile the 8 child octants as slots (the tree's child
         // table is the source table), Mc padded to square tables of Mt = max(S, R) rounded to 32,
@@ -459,9 +465,8 @@ int build_eval_data(Plan& p) {
                 if (np == 0) continue;
                 pad_mc<<<nbk(8LL * R * R, 256), 256, 0, st>>>(ptr<double>(op.Mc), S, p.R, R, ptr<double>(pad));
                 KF_LAUNCH();
-                KF_TRY(dev_alloc(op.Mhi, (size_t)m2l_tc_table_elems(R, 8) * 2));
-                KF_TRY(dev_alloc(op.Mlo, (size_t)m2l_tc_table_elems(R, 8) * 2));
-                KF_TRY(m2l_tc_prepare(st, ptr<double>(pad), R, op.Mhi.p, op.Mlo.p, &op.m2m_sT, 8));
+                KF_TRY(dev_alloc(op.Mtc, (size_t)m2l_tc_table_elems(R, 8) * 2));
+                KF_TRY(m2l_tc_prepare(st, ptr<double>(pad), R, op.Mtc.p, &op.m2m_sT, 8));
             }
             dev_free(pad);
             std::vector<int32_t> ms(std::max<size_t>(mt.size(), 1) * kSlotStride, 0);
@@ -472,13 +477,15 @@ int build_eval_data(Plan& p) {
             KF_TRY(dev_alloc(p.m2m_tiles, std::max<size_t>(mt.size(), 1) * sizeof(int4)));
             KF_TRY(dev_alloc(p.m2m_slots, ms.size() * 4));
             KF_TRY(dev_alloc(p.stage32, (size_t)nb * R * 4));
-            if (R > p.R) {
-                KF_TRY(dev_alloc(p.m2m_hi, (size_t)nb * R * 2));
-                KF_TRY(dev_alloc(p.m2m_lo, (size_t)nb * R * 2));
-            }
+            if (R > p.R) KF_TRY(dev_alloc(p.m2m_chl, (size_t)nb * R * 4));
             if (!mt.empty())
                 KF_CUDA(cudaMemcpyAsync(p.m2m_tiles.p, mt.data(), mt.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
             KF_CUDA(cudaMemcpyAsync(p.m2m_slots.p, ms.data(), ms.size() * 4, cudaMemcpyHostToDevice, st));
+            for (int l = 2; l + 1 < t.nlevels; ++l)
+                KF_TRY(tc_sched_build(st, ptr<int4>(p.m2m_tiles) + p.m2m_first[l], ptr<int32_t>(p.lv[l].parents),
+                                      ptr<int32_t>(t.child), 8,
+                                      ptr<int32_t>(p.m2m_slots) + (int64_t)p.m2m_first[l] * kSlotStride, p.m2m_count[l],
+                                      R, p.num_sms, p.sch_m2m[l]));
         }
         KF_CUDA(cudaStreamSynchronize(st));
     }
@@ -497,8 +504,7 @@ int build_eval_data(Plan& p) {
     }
     if (p.precision == KIFMM_MIXED) KF_TRY(dev_alloc(p.cu32, (size_t)nb * R * 4));
     if (p.m2l_tensor) {
-        KF_TRY(dev_alloc(p.chi, (size_t)nb * R * 2));
-        KF_TRY(dev_alloc(p.clo, (size_t)nb * R * 2));
+        KF_TRY(dev_alloc(p.chl, (size_t)nb * R * 4));
         KF_TRY(dev_alloc(p.cexp, (size_t)nb * 4));
     }
     if (p.lists[3].len > 0 && !p.cheb) KF_TRY(dev_alloc(p.chkx, (size_t)nb * S * ts));
@@ -1860,19 +1866,15 @@ static int run_far(Plan& p, const EvalView& E, int64_t& nl) {
             // before M2L), 8 octant slots per parent tile, staged in FP32, copied to the check rows
             const int64_t lo = t.level_start[l + 1], cnt = t.level_start[l + 2] - lo;
             const int Mt = p.m2m_R;
-            void* hi = Mt > R ? p.m2m_hi.p : p.chi.p;
-            void* lo16 = Mt > R ? p.m2m_lo.p : p.clo.p;
-            KF_TRY(m2l_tc_split_pad(st, cu + lo * R, cnt, R, Mt, static_cast<char*>(hi) + lo * Mt * 2,
-                                    static_cast<char*>(lo16) + lo * Mt * 2, ptr<int>(p.cexp) + lo));
+            char* chl = static_cast<char*>(Mt > R ? p.m2m_chl.p : p.chl.p);
+            KF_TRY(m2l_tc_split_pad(st, cu + lo * R, cnt, R, Mt, chl + lo * Mt * 4, ptr<int>(p.cexp) + lo));
             ++nl;
             M2LTables tabs{};
-            tabs.hi[l] = p.ops[l].Mhi.p;
-            tabs.lo[l] = p.ops[l].Mlo.p;
+            tabs.t[l] = p.ops[l].Mtc.p;
             tabs.sT[l] = p.ops[l].m2m_sT;
-            RUN(launch_tc_translate(st, tabs, Mt, ptr<int4>(p.m2m_tiles) + p.m2m_first[l], p.m2m_count[l],
-                                    ptr<int32_t>(LL.parents), ptr<int32_t>(t.child), 8,
-                                    ptr<int32_t>(p.m2m_slots) + (int64_t)p.m2m_first[l] * kSlotStride, hi, lo16,
-                                    ptr<int>(p.cexp), ptr<float>(p.stage32), 0, ptr<int>(p.err)));
+            KF_TRY(launch_tc_translate(st, tabs, Mt, p.sch_m2m[l], ptr<int4>(p.m2m_tiles) + p.m2m_first[l],
+                                       ptr<int32_t>(LL.parents), chl, ptr<int>(p.cexp), ptr<float>(p.stage32), 0,
+                                       ptr<int>(p.err), nl));
             rows_f2d<<<nbk((int64_t)LL.n_par * S, 256), 256, 0, st>>>(ptr<int32_t>(LL.parents), LL.n_par,
                                                                      ptr<float>(p.stage32), Mt,
                                                                      p.cheb ? cu : ptr<double>(p.chk),
@@ -1929,7 +1931,7 @@ static int run_far(Plan& p, const EvalView& E, int64_t& nl) {
         }
         c = reinterpret_cast<const T*>(ptr<float>(p.cu32));
         if (p.m2l_tensor) {
-            KF_TRY(m2l_tc_split(st, cu, t.nboxes, R, p.chi.p, p.clo.p, ptr<int>(p.cexp)));
+            KF_TRY(m2l_tc_split(st, cu, t.nboxes, R, p.chl.p, ptr<int>(p.cexp)));
             ++nl;
         }
     } else {
@@ -1938,15 +1940,12 @@ static int run_far(Plan& p, const EvalView& E, int64_t& nl) {
     if (sizeof(T) == 4 && p.m2l_tensor) {
         M2LTables tabs{};
         for (int l = 2; l < L; ++l) {
-            tabs.hi[l] = p.ops[l].Thi.p;
-            tabs.lo[l] = p.ops[l].Tlo.p;
+            tabs.t[l] = p.ops[l].Ttc.p;
             tabs.sT[l] = p.ops[l].tc_sT;
         }
         if (p.near_pending) KF_CUDA(cudaEventRecord(p.near_ev[0], st));   // (the near sums need q alone)
-        KF_TRY(launch_m2l_tc(st, tabs, R, ptr<int4>(p.tc_tiles), p.tc_ntiles, ptr<int32_t>(p.tc_boxes),
-                             ptr<int32_t>(p.vtab), ptr<int32_t>(p.tc_slots), p.chi.p, p.clo.p, ptr<int>(p.cexp),
-                             reinterpret_cast<float*>(dd), ptr<int>(p.err)));
-        ++nl;
+        KF_TRY(launch_tc_translate(st, tabs, R, p.sch_m2l, ptr<int4>(p.tc_tiles), ptr<int32_t>(p.tc_boxes), p.chl.p,
+                                   ptr<int>(p.cexp), reinterpret_cast<float*>(dd), 0, ptr<int>(p.err), nl));
         if (p.near_pending) KF_TRY(near_fork_launch(p, nl));
     } else {
         for (int l = 2; l < L; ++l) {
@@ -1989,17 +1988,14 @@ static int run_far(Plan& p, const EvalView& E, int64_t& nl) {
                 // by now), one slot per child octant, added onto the children's d
                 const int64_t lo = t.level_start[l - 1], cnt = t.level_start[l] - lo;
                 KF_TRY(m2l_tc_split_f32(st, reinterpret_cast<const float*>(dd) + lo * R, cnt, R,
-                                        static_cast<char*>(p.chi.p) + lo * R * 2, static_cast<char*>(p.clo.p) + lo * R * 2,
-                                        ptr<int>(p.cexp) + lo));
+                                        static_cast<char*>(p.chl.p) + lo * R * 4, ptr<int>(p.cexp) + lo));
                 ++nl;
                 M2LTables tabs{};
-                tabs.hi[l] = pop.Lhi.p;
-                tabs.lo[l] = pop.Llo.p;
+                tabs.t[l] = pop.Ltc.p;
                 tabs.sT[l] = pop.l2l_sT;
-                RUN(launch_tc_translate(st, tabs, R, ptr<int4>(p.tc_tiles) + p.tc_first[l], p.tc_count[l],
-                                        ptr<int32_t>(p.tc_boxes), ptr<int32_t>(p.ptab), 8,
-                                        ptr<int32_t>(p.l2l_slots) + (int64_t)p.tc_first[l] * kSlotStride, p.chi.p,
-                                        p.clo.p, ptr<int>(p.cexp), reinterpret_cast<float*>(dd), 1, ptr<int>(p.err)));
+                KF_TRY(launch_tc_translate(st, tabs, R, p.sch_l2l[l], ptr<int4>(p.tc_tiles) + p.tc_first[l],
+                                           ptr<int32_t>(p.tc_boxes), p.chl.p, ptr<int>(p.cexp),
+                                           reinterpret_cast<float*>(dd), 1, ptr<int>(p.err), nl));
             } else if (LP.l2l_max > 0 && sizeof(T) == 4 && op.rank <= MM_TM && pop.rank <= MM_NS * MM_TK) {
                 // FP32, one block per (octant, tile of parents), every chunk loaded at once (32
                 // parents a tile where that gives every SM two blocks, else 16)
@@ -2096,8 +2092,8 @@ int run_eval(Plan& p, const void* I, void* S_out, int dtype, double C) {
         // Chebyshev: the W list reads the node weights c (stride R) and the local part
         // interpolates d in a second kernel
         if (p.lat_far && !p.cheb && t.nlevels > 2) {   // uniform lattice, no W list: the local part is one matrix from d
-            KF_TRY(lat_l2p(p));
-            if (p.lat_l2p_tc) ++nl;   // (the split of d, then the translation kernel)
+            KF_TRY(lat_l2p(p, nl));
+            --nl;   // (counted below)
         } else if (mixed) {
             auto* kl2p = p.far_series ? k_l2p<true, true, float> : k_l2p<true, false, float>;
             kl2p<<<(unsigned)p.nleaves, L2P_T, 0, st>>>(E, ptr<int32_t>(p.leaves), wo, wi, ptr<float>(p.phid),

@@ -70,6 +70,14 @@ struct AllocFaultScope {
 void dev_free(DevBuf& b);
 template <class T> T* ptr(const DevBuf& b) { return reinterpret_cast<T*>(b.p); }
 
+// Split of one tensor-core translation launch over the SMs (m2l_tc.cu): prefix sums of the tiles'
+// slot counts, the CTAs, and the work space for the pieces of the tiles that are cut between CTAs
+struct TcSched {
+    int ntiles = 0, total = 0, ncta = 0;
+    bool finish = false;   // some tile is cut, or has no slot
+    DevBuf pre, first, src, meta, part;
+};
+
 // ---- plan ---------------------------------------------------------------------------
 struct Tree {
     int64_t n = 0;          // points
@@ -112,14 +120,14 @@ struct LevelOps {
     DevBuf Lo;           // [8][R][R] L2L in coefficients, parent level = this level
     // FP32 copies (mixed form)
     DevBuf T32, Ub32, Vb32, Vt32, Lo32, Mc32;
-    // tensor-core M2L operands: FP16 hi/lo of T 2^tc_sT, [slot][k-chunk][row][128-byte swizzled row]
-    DevBuf Thi, Tlo;
+    // tensor-core M2L operand: FP16 hi / lo of T 2^tc_sT, [slot][k-chunk][row][128-byte swizzled row]
+    DevBuf Ttc;
     int tc_sT = 0;
     // tensor-core L2L (parent level = this level): FP16 hi/lo of Lo 2^l2l_sT, 8 slots
-    DevBuf Lhi, Llo;
+    DevBuf Ltc;
     int l2l_sT = 0;
     // tensor-core M2M translations (parent level = this level): FP16 hi/lo of Mc (rows padded to R)
-    DevBuf Mhi, Mlo;
+    DevBuf Mtc;
     int m2m_sT = 0;
     // FP64-exact upward solve on the tensor cores: integer slices of G1 (swizzled images) and
     // the per-row power-of-two exponents
@@ -160,8 +168,8 @@ struct Plan {
     DevBuf chkx;       // T[nb*S]  downward check potentials from the X list (S2L)
     DevBuf cu;         // f64[nb*R] upward coefficients c
     DevBuf cu32;       // f32[nb*R] (mixed) FP32 copy of c for the SIMT M2L and the W list
-    DevBuf chi, clo;   // f16[nb*R] (mixed, tensor-core M2L) hi/lo parts of c 2^cexp
-    DevBuf cexp;       // i32[nb] per-box power-of-two scale of chi/clo
+    DevBuf chl;        // f16[nb*2R] (mixed, tensor-core M2L) c 2^cexp, per 32 columns 32 hi then 32 lo parts
+    DevBuf cexp;       // i32[nb] per-box power-of-two scale of chl
     DevBuf dd;         // T[nb*R]  downward coefficients d
     DevBuf phid;       // T[nb*S]  downward equivalent densities of the leaves
     DevBuf phiu;       // T[nb*S]  upward equivalent densities (only when W lists exist)
@@ -196,7 +204,7 @@ struct Plan {
     DevBuf m2m_tiles, m2m_slots, stage32;   // parent tiles per level, their 8 slots, FP32 staging [nb][m2m_R]
     DevBuf apply_part;                      // partial sums of the SIMT applies split over their terms
     int m2m_R = 0;                          // square table size of the M2M translations: max(S, R) rounded to 32
-    DevBuf m2m_hi, m2m_lo;                  // children's c split FP16 x 2 in rows of m2m_R (when m2m_R > R)
+    DevBuf m2m_chl;                         // children's c split FP16 x 2 in rows of m2m_R (when m2m_R > R)
     int m2m_first[kMaxLevel + 1] = {0}, m2m_count[kMaxLevel + 1] = {0};
     int num_sms = 1;             // multiprocessors of the plan's device (grid sizing)
     bool p2p_series = true;      // some near pair is closer than 0.5 / (b - a) (mixed P2P)
@@ -209,12 +217,12 @@ struct Plan {
     // near field on the tensor cores (mixed form, uniform lattice; near_tc.cu)
     bool near_tc = false;
     int nf_R = 0, nf_level = 0, nf_sT = 0, nf_ntiles = 0;
-    DevBuf nf_utab, nf_Thi, nf_Tlo, nf_tiles, nf_slots, nf_boxes, nf_qhi, nf_qlo, nf_qexp, nf_near, nf_ref;
+    DevBuf nf_utab, nf_Ttc, nf_tiles, nf_slots, nf_boxes, nf_qhl, nf_qexp, nf_near, nf_ref;
     bool lat_far = false;        // S2M and local L2P on the same lattice (surface form, no W / X lists)
     DevBuf lat_P;                // f32 [S][npl + 1]: K between the leaf's check surface and its cells
     DevBuf lat_Q;                // f32 [R][npl + 1]: P^T Ub, the leaf's local expansion from its coefficients d
     bool lat_l2p_tc = false;     // that expansion through the tensor-core kernel (FP32 rows in lat_fst)
-    DevBuf lat_Thi, lat_Tlo, lat_iota, lat_slots, lat_fst;
+    DevBuf lat_Ttc, lat_iota, lat_slots, lat_fst;
     int lat_sT = 0;
     bool lat_up = false;         // leaves' c = (G1 P) q on the tensor cores, FP64-exact (no leaf S2M)
     DevBuf lat_Mimg, lat_Mer;    // slice image and row exponents of M = G1 P (rank x npl)
@@ -227,6 +235,7 @@ struct Plan {
     DevBuf tc_boxes;             // boxes of every level grouped by octant, level after level
     DevBuf tc_slots;             // [tile][344] active offset slots
     int tc_ntiles = 0;
+    TcSched sch_m2l, sch_near, sch_lat, sch_l2l[kMaxLevel + 1], sch_m2m[kMaxLevel + 1];
     DevBuf err;                  // int: device-side error code (bounded waits)
     int64_t p2p_pairs = 0;       // near-field pairs of one evaluation
     double m2l_flops = 0;        // algorithmic M2L flop of one evaluation (2 r^2 per V pair)
@@ -273,32 +282,31 @@ int build_operators(Plan& p);
 int build_self_terms(Plan& p, const double* h_dev, double uniform_h);
 // m2l_tc.cu
 int m2l_tc_supported(int R);
-int64_t m2l_tc_table_elems(int R, int nslots = kOffsetSlots);   // FP16 elements of one level's Thi (or Tlo)
-int m2l_tc_prepare(cudaStream_t st, const double* T, int R, void* Thi, void* Tlo, int* sT_out,
-                   int nslots = kOffsetSlots);
-int m2l_tc_split(cudaStream_t st, const double* c, int64_t nb, int R, void* chi, void* clo, int* cexp);
-// the same with output rows of ldo >= R halves (columns R..ldo-1 zero)
-int m2l_tc_split_pad(cudaStream_t st, const double* c, int64_t nb, int R, int ldo, void* chi, void* clo, int* cexp);
-int m2l_tc_split_f32(cudaStream_t st, const float* c, int64_t nb, int R, void* chi, void* clo, int* cexp);
-struct M2LTables {                 // per-level FP16 hi/lo M2L tables for the tensor-core kernel
-    const void* hi[kMaxLevel + 1];
-    const void* lo[kMaxLevel + 1];
+int64_t m2l_tc_table_elems(int R, int nslots = kOffsetSlots);   // FP16 elements (hi and lo) of one level's table
+int m2l_tc_prepare(cudaStream_t st, const double* T, int R, void* out, int* sT_out, int nslots = kOffsetSlots);
+int m2l_tc_split(cudaStream_t st, const double* c, int64_t nb, int R, void* out, int* cexp);
+// the same with output rows of ldo >= R columns (columns R..ldo-1 zero)
+int m2l_tc_split_pad(cudaStream_t st, const double* c, int64_t nb, int R, int ldo, void* out, int* cexp);
+int m2l_tc_split_f32(cudaStream_t st, const float* c, int64_t nb, int R, void* out, int* cexp);
+struct M2LTables {                 // per-level FP16 hi/lo tables for the tensor-core kernel
+    const void* t[kMaxLevel + 1];
     int sT[kMaxLevel + 1];         // the tables hold T 2^sT
 };
-int launch_m2l_tc(cudaStream_t st, const M2LTables& tabs, int R, const int4* tiles, int ntiles, const int32_t* boxes,
-                  const int32_t* vtab, const int32_t* slots, const void* chi, const void* clo, const int* cexp, float* d,
-                  int* err);
-// the same kernel with any source table stride (nslots slots per target box) and, with
-// accum != 0, the result added to d (L2L onto the M2L result)
-int launch_tc_translate(cudaStream_t st, const M2LTables& tabs, int R, const int4* tiles, int ntiles,
-                        const int32_t* boxes, const int32_t* vtab, int vstride, const int32_t* slots, const void* chi,
-                        const void* clo, const int* cexp, float* d, int accum, int* err);
+// the split of the tiles (level, first box in boxes, box count) whose slot lists are at `slots`,
+// their sources taken from the table vtab of vstride entries per target box (plan time)
+int tc_sched_build(cudaStream_t st, const int4* tiles, const int32_t* boxes, const int32_t* vtab, int vstride,
+                   const int32_t* slots, int ntiles, int R, int num_sms, TcSched& s);
+// d[B] = sum over the tile's slots of T[slot] c[source(B, slot)] (chl, cexp: the split rows of c), or
+// added to d with accum != 0 (L2L onto the M2L result); nl += the launches
+int launch_tc_translate(cudaStream_t st, const M2LTables& tabs, int R, const TcSched& sched, const int4* tiles,
+                        const int32_t* boxes, const void* chl, const int* cexp, float* d, int accum, int* err,
+                        int64_t& nl);
 // near_tc.cu: near field on a uniform lattice
 int near_tc_plan(Plan& p);
 int near_tc_contract(Plan& p, cudaStream_t st, int64_t& nl);   // the near sums into nf_near on st
 int near_tc_finish(Plan& p, const double* far, double C, void* out, int dtype, int64_t& nl);
 int lat_s2m(Plan& p);   // chk of every leaf (lat_far plans)
-int lat_l2p(Plan& p);   // far of every point from the leaves' d (lat_far plans)
+int lat_l2p(Plan& p, int64_t& nl);   // far of every point from the leaves' d (lat_far plans)
 int lat_up_plan(Plan& p);   // M = G1 P for the leaves' FP64-exact upward solve (after the slice set-up)
 int lat_up_apply(Plan& p, double* cu, int64_t& nl);   // c of every leaf = M q
 // pinv_oz.cu: FP64-exact c = Sigma^+ U^T chk on the tensor cores

@@ -323,20 +323,19 @@ int lat_s2m(Plan& p) {   // surface form: check potentials; Chebyshev: node weig
     return KIFMM_OK;
 }
 
-int lat_l2p(Plan& p) {
+int lat_l2p(Plan& p, int64_t& nl) {
     if (p.lat_l2p_tc) {   // tensor cores: the leaves' d split FP16 x 3, one slot (the leaf itself)
         cudaStream_t st = p.stream;
         const int R = p.R, lf = p.nf_level;
         const int64_t lo = p.tree.level_start[lf], cnt = p.tree.level_start[lf + 1] - lo;
-        KF_TRY(m2l_tc_split_f32(st, ptr<float>(p.dd) + lo * R, cnt, R, static_cast<char*>(p.chi.p) + lo * R * 2,
-                                static_cast<char*>(p.clo.p) + lo * R * 2, ptr<int>(p.cexp) + lo));
+        KF_TRY(m2l_tc_split_f32(st, ptr<float>(p.dd) + lo * R, cnt, R, static_cast<char*>(p.chl.p) + lo * R * 4,
+                                ptr<int>(p.cexp) + lo));
         M2LTables tabs{};
-        tabs.hi[lf] = p.lat_Thi.p;
-        tabs.lo[lf] = p.lat_Tlo.p;
+        tabs.t[lf] = p.lat_Ttc.p;
         tabs.sT[lf] = p.lat_sT;
-        return launch_tc_translate(st, tabs, R, ptr<int4>(p.nf_tiles), p.nf_ntiles, ptr<int32_t>(p.leaves),
-                                   ptr<int32_t>(p.lat_iota), 1, ptr<int32_t>(p.lat_slots), p.chi.p, p.clo.p,
-                                   ptr<int>(p.cexp), ptr<float>(p.lat_fst), 0, ptr<int>(p.err));
+        ++nl;
+        return launch_tc_translate(st, tabs, R, p.sch_lat, ptr<int4>(p.nf_tiles), ptr<int32_t>(p.leaves), p.chl.p,
+                                   ptr<int>(p.cexp), ptr<float>(p.lat_fst), 0, ptr<int>(p.err), nl);
     }
     const int lpp = LT_T / p.nf_R * LT_LT;
     const unsigned g = (unsigned)std::min<int64_t>((p.nleaves + lpp - 1) / lpp, 8LL * p.num_sms);
@@ -344,6 +343,7 @@ int lat_l2p(Plan& p) {
                                                                 ptr<int32_t>(p.leaves), p.nleaves, ptr<float>(p.dd),
                                                                 ptr<double>(p.far));
     KF_LAUNCH();
+    ++nl;
     return KIFMM_OK;
 }
 
@@ -429,9 +429,8 @@ int near_tc_plan(Plan& p) {
     KF_CUDA(cudaMemsetAsync(T.p, 0, kOffsetSlots * RR * 8, st));
     k_nf_table<<<nbn(27 * RR, 256), 256, 0, st>>>(ptr<int32_t>(ref), nc, R, h, make_kparams_kind(p.kind, p.a, p.b), ptr<double>(T));
     KF_LAUNCH();
-    KF_TRY(dev_alloc(p.nf_Thi, (size_t)m2l_tc_table_elems(R) * 2));
-    KF_TRY(dev_alloc(p.nf_Tlo, (size_t)m2l_tc_table_elems(R) * 2));
-    KF_TRY(m2l_tc_prepare(st, ptr<double>(T), R, p.nf_Thi.p, p.nf_Tlo.p, &p.nf_sT));
+    KF_TRY(dev_alloc(p.nf_Ttc, (size_t)m2l_tc_table_elems(R) * 2));
+    KF_TRY(m2l_tc_prepare(st, ptr<double>(T), R, p.nf_Ttc.p, &p.nf_sT));
     // S2M (P2M) and local L2P on the lattice: leaves at level >= 2, no W / X lists. Surface
     // form: the check matrix P and Q = P^T U Sigma^+; Chebyshev form: the interpolation
     // weights S3(xbar_m, u_i) of the leaf's cells for P2M (its L2P keeps the interpolation
@@ -480,9 +479,8 @@ int near_tc_plan(Plan& p) {
                                                                     p.r_out, h,
                                                                     make_kparams_kind(p.kind, p.a, p.b), ptr<double>(QT));
             KF_LAUNCH();
-            KF_TRY(dev_alloc(p.lat_Thi, (size_t)m2l_tc_table_elems(p.R, 1) * 2));
-            KF_TRY(dev_alloc(p.lat_Tlo, (size_t)m2l_tc_table_elems(p.R, 1) * 2));
-            KF_TRY(m2l_tc_prepare(st, ptr<double>(QT), p.R, p.lat_Thi.p, p.lat_Tlo.p, &p.lat_sT, 1));
+            KF_TRY(dev_alloc(p.lat_Ttc, (size_t)m2l_tc_table_elems(p.R, 1) * 2));
+            KF_TRY(m2l_tc_prepare(st, ptr<double>(QT), p.R, p.lat_Ttc.p, &p.lat_sT, 1));
             KF_TRY(dev_alloc(p.lat_iota, (size_t)t.nboxes * 4));
             k_iota<<<nbn(t.nboxes, 256), 256, 0, st>>>(ptr<int32_t>(p.lat_iota), t.nboxes);
             KF_LAUNCH();
@@ -518,8 +516,12 @@ int near_tc_plan(Plan& p) {
     KF_CUDA(cudaMemcpyAsync(p.nf_tiles.p, tiles.data(), tiles.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
     KF_CUDA(cudaMemcpyAsync(p.nf_slots.p, slots.data(), slots.size() * 4, cudaMemcpyHostToDevice, st));
     KF_CUDA(cudaMemcpyAsync(p.nf_boxes.p, ids.data(), ids.size() * 4, cudaMemcpyHostToDevice, st));
-    KF_TRY(dev_alloc(p.nf_qhi, (size_t)n * 2));
-    KF_TRY(dev_alloc(p.nf_qlo, (size_t)n * 2));
+    KF_TRY(tc_sched_build(st, ptr<int4>(p.nf_tiles), ptr<int32_t>(p.nf_boxes), ptr<int32_t>(p.nf_utab), kOffsetSlots,
+                          ptr<int32_t>(p.nf_slots), ntiles, R, p.num_sms, p.sch_near));
+    if (p.lat_l2p_tc)
+        KF_TRY(tc_sched_build(st, ptr<int4>(p.nf_tiles), ptr<int32_t>(p.leaves), ptr<int32_t>(p.lat_iota), 1,
+                              ptr<int32_t>(p.lat_slots), ntiles, p.R, p.num_sms, p.sch_lat));
+    KF_TRY(dev_alloc(p.nf_qhl, (size_t)n * 4));
     KF_TRY(dev_alloc(p.nf_qexp, (size_t)nl * 4));
     KF_TRY(dev_alloc(p.nf_near, (size_t)n * 4));
     KF_CUDA(cudaStreamSynchronize(st));
@@ -600,16 +602,13 @@ int lat_up_apply(Plan& p, double* cu, int64_t& nl) {
 // the per-offset contractions of the near field into nf_near, on stream st (they read only the
 // sorted weights q)
 int near_tc_contract(Plan& p, cudaStream_t st, int64_t& nl) {
-    KF_TRY(m2l_tc_split(st, ptr<double>(p.q), p.nleaves, p.nf_R, p.nf_qhi.p, p.nf_qlo.p, ptr<int>(p.nf_qexp)));
+    KF_TRY(m2l_tc_split(st, ptr<double>(p.q), p.nleaves, p.nf_R, p.nf_qhl.p, ptr<int>(p.nf_qexp)));
     ++nl;
     M2LTables tabs{};
-    tabs.hi[p.nf_level] = p.nf_Thi.p;
-    tabs.lo[p.nf_level] = p.nf_Tlo.p;
+    tabs.t[p.nf_level] = p.nf_Ttc.p;
     tabs.sT[p.nf_level] = p.nf_sT;
-    KF_TRY(launch_m2l_tc(st, tabs, p.nf_R, ptr<int4>(p.nf_tiles), p.nf_ntiles, ptr<int32_t>(p.nf_boxes),
-                         ptr<int32_t>(p.nf_utab), ptr<int32_t>(p.nf_slots), p.nf_qhi.p, p.nf_qlo.p, ptr<int>(p.nf_qexp),
-                         ptr<float>(p.nf_near), ptr<int>(p.err)));
-    ++nl;
+    KF_TRY(launch_tc_translate(st, tabs, p.nf_R, p.sch_near, ptr<int4>(p.nf_tiles), ptr<int32_t>(p.nf_boxes), p.nf_qhl.p,
+                               ptr<int>(p.nf_qexp), ptr<float>(p.nf_near), 0, ptr<int>(p.err), nl));
     return KIFMM_OK;
 }
 
