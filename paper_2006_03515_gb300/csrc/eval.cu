@@ -11,6 +11,7 @@
 #include "internal.cuh"
 #include "cheb.cuh"
 #include "kernel.cuh"
+#include "pair64.cuh"
 
 namespace kifmm {
 
@@ -34,6 +35,13 @@ __global__ void local_coords(const double* spts, const int32_t* leaf_of, const d
     const double* c = centre + 3 * (int64_t)leaf_of[k];
     loc[k] = make_float4((float)(spts[3 * k] - c[0]), (float)(spts[3 * k + 1] - c[1]),
                          (float)(spts[3 * k + 2] - c[2]), 0.f);
+}
+
+__global__ void k_p64_table(double* out) {
+    __shared__ Pair64Tab tab;
+    pair64_tab_fill(tab);
+    __syncthreads();
+    for (int e = threadIdx.x; e < 2 * kPairTab; e += blockDim.x) out[e] = tab.t[e];
 }
 
 __global__ void select_boxes(const int32_t* level, const int32_t* leaf, int64_t lo, int64_t hi,
@@ -198,6 +206,10 @@ int build_eval_data(Plan& p) {
     KF_TRY(dev_alloc(p.loc32, n * sizeof(float4)));
     local_coords<<<nbk(n, 256), 256, 0, st>>>(ptr<double>(p.pts), ptr<int32_t>(p.leaf_of),
                                               ptr<double>(t.centre), n, ptr<float4>(p.loc32));
+    KF_LAUNCH();
+
+    KF_TRY(dev_alloc(p.p64tab, sizeof(Pair64Tab)));
+    k_p64_table<<<1, 256, 0, st>>>(ptr<double>(p.p64tab));
     KF_LAUNCH();
 
     DevBuf flag, pos, scan_tmp;
@@ -567,8 +579,18 @@ struct EvalView {
     int cp;                 // Chebyshev order p
     const double* ctab;     // Chebyshev weight table c_k T_k(xbar_n), row stride kChebTab
     const float* ctab32;
+    Pair64 p64;             // FP64 pair loops of the paper's kernel (kind 0), with their table
+    const double* p64tab;
     int64_t n_real;         // the caller's points (sorted points with perm >= n_real are padding cells)
 };
+
+// the FP64 kernel of one pair, and its table brought into the block's shared memory
+__device__ __forceinline__ void p64_load(const EvalView& E, Pair64Tab& tab) {
+    for (int e = threadIdx.x; e < 2 * kPairTab; e += blockDim.x) tab.t[e] = E.p64tab[e];
+}
+__device__ __forceinline__ double p64_pair(double r2, const EvalView& E, const Pair64Tab& tab) {
+    return E.kp.kind ? kern_f64(sqrt(r2), E.kp) : pair64_kernel(r2, E.p64, tab);
+}
 
 __device__ __forceinline__ double half_width(const EvalView& E, int lev) {
     return E.side / (double)(2ll << lev);
@@ -604,6 +626,8 @@ __global__ void __launch_bounds__(P2M_T) k_p2m(EvalView E, const int32_t* boxes,
     const int p0 = E.pstart[B], p1 = E.pend[B];
     __shared__ float4 sp32[256];
     __shared__ double sp64[256][4];
+    __shared__ Pair64Tab tab;
+    if (!MIXED) p64_load(E, tab);
     const double* c = E.centre + 3 * (int64_t)B;
     for (int j0 = 0; j0 < S; j0 += P2M_T) {
         const int j = j0 + threadIdx.x;
@@ -648,7 +672,7 @@ __global__ void __launch_bounds__(P2M_T) k_p2m(EvalView E, const int32_t* boxes,
             } else {
                 for (int e = 0; e < ns; ++e) {
                     const double dx = xj[0] - sp64[e][0], dy = xj[1] - sp64[e][1], dz = xj[2] - sp64[e][2];
-                    acc64 += kern_f64(sqrt(dx * dx + dy * dy + dz * dz), E.kp) * sp64[e][3];
+                    acc64 += p64_pair(dx * dx + dy * dy + dz * dz, E, tab) * sp64[e][3];
                 }
             }
         }
@@ -1101,6 +1125,8 @@ __global__ void __launch_bounds__(P2M_T) k_s2l_x(EvalView E, const int32_t* boxe
     const double* cB = E.centre + 3 * (int64_t)B;
     __shared__ float4 sp32[256];
     __shared__ double sp64[256][4];
+    __shared__ Pair64Tab tab;
+    if (!MIXED) p64_load(E, tab);
     for (int j0 = 0; j0 < S; j0 += P2M_T) {
         const int j = j0 + threadIdx.x;
         double xj[3];
@@ -1134,7 +1160,7 @@ __global__ void __launch_bounds__(P2M_T) k_s2l_x(EvalView E, const int32_t* boxe
                 } else {
                     for (int e = 0; e < ns; ++e) {
                         const double dx = xj[0] - sp64[e][0], dy = xj[1] - sp64[e][1], dz = xj[2] - sp64[e][2];
-                        acc64 += kern_f64(sqrt(dx * dx + dy * dy + dz * dz), E.kp) * sp64[e][3];
+                        acc64 += p64_pair(dx * dx + dy * dy + dz * dz, E, tab) * sp64[e][3];
                     }
                 }
             }
@@ -1163,6 +1189,8 @@ __global__ void __launch_bounds__(L2P_T) k_l2p(EvalView E, const int32_t* leaves
     const double* cB = E.centre + 3 * (int64_t)B;
     __shared__ float4 s32[320];
     __shared__ double s64[320][4];
+    __shared__ Pair64Tab tab;
+    if (!MIXED) p64_load(E, tab);
     const int p0 = E.pstart[B], p1 = E.pend[B];
     const int nsrc_lists = 1 + (woff[B + 1] - woff[B]);
     for (int t0 = p0; t0 < p1; t0 += L2P_T) {
@@ -1229,7 +1257,7 @@ __global__ void __launch_bounds__(L2P_T) k_l2p(EvalView E, const int32_t* leaves
                 } else {
                     for (int e = 0; e < ns; ++e) {
                         const double dx = x64[0] - s64[e][0], dy = x64[1] - s64[e][1], dz = x64[2] - s64[e][2];
-                        acc64 += kern_f64(sqrt(dx * dx + dy * dy + dz * dz), E.kp) * s64[e][3];
+                        acc64 += p64_pair(dx * dx + dy * dy + dz * dz, E, tab) * s64[e][3];
                     }
                 }
             }
@@ -1451,6 +1479,8 @@ __global__ void __launch_bounds__(P2P_T) k_p2p(EvalView E, const int32_t* leaves
     float4* s32 = reinterpret_cast<float4*>(smem_raw);
     double* s64 = reinterpret_cast<double*>(smem_raw);
     __shared__ double red[P2P_GRP][P2P_TGT];
+    __shared__ Pair64Tab tab;
+    if (!MIXED) p64_load(E, tab);
     const int p0 = E.pstart[B], p1 = E.pend[B];
     const int tl = threadIdx.x % P2P_TGT, g = threadIdx.x / P2P_TGT;
     const int u0 = uoff[B], u1 = uoff[B + 1];
@@ -1513,7 +1543,7 @@ __global__ void __launch_bounds__(P2P_T) k_p2p(EvalView E, const int32_t* leaves
                         const double dx = x64[0] - s64[4 * e], dy = x64[1] - s64[4 * e + 1],
                                      dz = x64[2] - s64[4 * e + 2];
                         const double r2 = dx * dx + dy * dy + dz * dz;
-                        if (r2 > 0.0) acc64 += kern_f64(sqrt(r2), E.kp) * s64[4 * e + 3];
+                        if (r2 > 0.0) acc64 += p64_pair(r2, E, tab) * s64[4 * e + 3];
                     }
                 }
             }
@@ -1702,6 +1732,8 @@ static EvalView make_view(Plan& p) {
     E.ctab = ptr<double>(p.ctab);
     E.ctab32 = ptr<float>(p.ctab32);
     E.n_real = p.n_real;
+    E.p64 = make_pair64(E.kp);
+    E.p64tab = ptr<double>(p.p64tab);
     return E;
 }
 

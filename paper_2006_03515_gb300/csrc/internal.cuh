@@ -147,6 +147,7 @@ struct Plan {
     Csr lists[4];                 // U, V, W, X
     DevBuf vtab;                  // i32[nb * 343]: source box of V(B) at offset slot, -1 if none
     std::vector<LevelOps> ops;    // indexed by level (entries below 2 unused)
+    DevBuf p64tab;                // exponential tables of the FP64 pair kernel (pair64.cuh)
     DevBuf surf;                  // f64[3*S] unit lattice (Chebyshev representation: the p^3 nodes)
     DevBuf ctab, ctab32;          // f64 / f32 [p][10]: c_k T_k(node_n), c_0 = 1/p, c_k = 2/p (Chebyshev only)
     DevBuf cheb_A;                // f64 [2][p][p]: 1-D factors of the M2M / L2L interpolation (Chebyshev only)
