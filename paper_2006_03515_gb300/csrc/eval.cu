@@ -1979,6 +1979,16 @@ static int run_far(Plan& p, const EvalView& E, int64_t& nl) {
         KF_TRY(launch_tc_translate(st, tabs, R, p.sch_m2l, ptr<int4>(p.tc_tiles), ptr<int32_t>(p.tc_boxes), p.chl.p,
                                    ptr<int>(p.cexp), reinterpret_cast<float*>(dd), 0, ptr<int>(p.err), nl));
         if (p.near_pending) KF_TRY(near_fork_launch(p, nl));
+    } else if (p.fft_m2l) {   // FP64 form: phi = V c, the transforms, d = V^T q
+        double* fq = ptr<double>(p.fft_q);
+        for (int l = 2; l < L; ++l)
+            RUN(launch_apply<double>(st, ptr<double>(p.ops[l].Vb), R, S, p.ops[l].rank, nullptr, nullptr,
+                                     t.level_start[l], (int)(t.level_start[l + 1] - t.level_start[l]), cu, R, fq, S, 0));
+        KF_TRY(fft_m2l_apply(p, nl));
+        for (int l = 2; l < L; ++l)
+            RUN(launch_apply<double>(st, ptr<double>(p.ops[l].Vt), S, p.ops[l].rank, S, nullptr, nullptr,
+                                     t.level_start[l], (int)(t.level_start[l + 1] - t.level_start[l]), fq, S,
+                                     reinterpret_cast<double*>(dd), R, 0));
     } else {
         for (int l = 2; l < L; ++l) {
             auto& LL = p.lv[l];

@@ -236,6 +236,9 @@ struct Plan {
     DevBuf tc_boxes;             // boxes of every level grouped by octant, level after level
     DevBuf tc_slots;             // [tile][344] active offset slots
     int tc_ntiles = 0;
+    bool fft_m2l = false;        // FP64 form: M2L by Fourier transforms (fft_m2l.cu)
+    DevBuf fft_idx, fft_tab, fft_spec, fft_q;   // lattice point -> surface point; [level - 2][343] kernel
+                                                // transforms; box spectra; [box][S] densities, then potentials
     TcSched sch_m2l, sch_near, sch_lat, sch_l2l[kMaxLevel + 1], sch_m2m[kMaxLevel + 1];
     DevBuf err;                  // int: device-side error code (bounded waits)
     int64_t p2p_pairs = 0;       // near-field pairs of one evaluation
@@ -302,6 +305,10 @@ int tc_sched_build(cudaStream_t st, const int4* tiles, const int32_t* boxes, con
 int launch_tc_translate(cudaStream_t st, const M2LTables& tabs, int R, const TcSched& sched, const int4* tiles,
                         const int32_t* boxes, const void* chl, const int* cexp, float* d, int accum, int* err,
                         int64_t& nl);
+// fft_m2l.cu: M2L of the FP64 form by Fourier transforms
+bool fft_m2l_wanted(const Plan& p);
+int fft_m2l_plan(Plan& p);
+int fft_m2l_apply(Plan& p, int64_t& nl);
 // near_tc.cu: near field on a uniform lattice
 int near_tc_plan(Plan& p);
 int near_tc_contract(Plan& p, cudaStream_t st, int64_t& nl);   // the near sums into nf_near on st

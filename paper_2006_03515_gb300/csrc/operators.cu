@@ -474,7 +474,9 @@ int build_operators(Plan& p) {
     KF_TRY(dev_alloc(m2l, kOffsetSlots * SS * 8));
     KF_TRY(dev_alloc(w, kOffsetSlots * SR * 8));
     std::vector<double> sh(kOffsetSlots * 3);
-    for (int l = 2; l < L; ++l) {
+    const bool fft = fft_m2l_wanted(p);   // (then no dense tables)
+    if (fft) KF_TRY(fft_m2l_plan(p));
+    for (int l = 2; l < L && !fft; ++l) {
         LevelOps& op = p.ops[l];
         double r = op.r;
         for (int dz = -3; dz <= 3; ++dz)
