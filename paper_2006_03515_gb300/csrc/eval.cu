@@ -531,7 +531,8 @@ int build_eval_data(Plan& p) {
     // FP64-exact upward solves on the tensor cores (mixed form; KIFMM_UPWARD=fp64 keeps the FP64 pipe)
     {
         const char* up = std::getenv("KIFMM_UPWARD");
-        p.oz = p.precision == KIFMM_MIXED && !p.cheb && pinv_oz_supported(S) && !(up && std::string(up) == "fp64");
+        p.oz_any = p.precision == KIFMM_MIXED && !p.cheb && !(up && std::string(up) == "fp64");
+        p.oz = p.oz_any && pinv_oz_supported(S);
         const char* om = std::getenv("KIFMM_OZ_MIN");   // level-size threshold (tests use 0)
         p.oz_min = om ? std::max(0, std::atoi(om)) : kOzMinBoxes;
         // smallest tile count of a level whose M2M / L2L take the tensor-core translation

@@ -229,6 +229,7 @@ struct Plan {
     DevBuf lat_Mimg, lat_Mer;    // slice image and row exponents of M = G1 P (rank x npl)
     bool far_series = true;      // likewise for a leaf's points and its check / equivalent surfaces
     bool oz = false;             // upward pseudo-inverse by exact slicing on the tensor cores (mixed form)
+    bool oz_any = false;         // exact slicing may be used where the operator fits (oz: it does for S columns)
     DevBuf ozBox, ozEb;          // per-level work space: box slice images, box exponents
     int oz_min = kOzMinBoxes;    // levels with more upward solves than this use the slice products
     int tc_min_tiles = kTcMinTiles;   // levels with at least this many tiles: tensor-core M2M / L2L

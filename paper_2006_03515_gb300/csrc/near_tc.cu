@@ -568,7 +568,10 @@ __global__ void k_lat_M(const double* G1, int S, int rank, const double* surf, c
 int lat_up_plan(Plan& p) {
     p.lat_up = false;
     const int lf = p.nf_level, npl = p.nf_R;
-    if (!p.lat_far || !p.oz || lf < 2 || lf >= p.tree.nlevels || p.nleaves <= p.oz_min) return KIFMM_OK;
+    // (K = npl = 64 here, whatever S: surface orders whose S-column operator does not fit the slice
+    // kernel's shared memory, m0 >= 8, take it for their leaves too. At 101^3 padded, m0 = 8, the 17576
+    // leaves' check potentials and FP64 product took 1.37 ms, this takes 69 us.)
+    if (!p.lat_far || !p.oz_any || lf < 2 || lf >= p.tree.nlevels || p.nleaves <= p.oz_min) return KIFMM_OK;
     if (p.lv[lf].n_par != 0 || p.lv[lf].n_up != p.nleaves || !pinv_oz_supported(npl)) return KIFMM_OK;
     cudaStream_t st = p.stream;
     const LevelOps& op = p.ops[lf];
@@ -584,6 +587,10 @@ int lat_up_plan(Plan& p) {
     KF_TRY(dev_alloc(p.lat_Mimg, pinv_oz_op_bytes(npl, op.rank)));
     KF_TRY(dev_alloc(p.lat_Mer, (size_t)((op.rank + 47) / 48 * 48) * 4));
     KF_TRY(pinv_oz_prepare(st, ptr<double>(M), npl, op.rank, p.lat_Mimg.p, ptr<int>(p.lat_Mer)));
+    if (!p.oz) {   // (else the level work space, at least as large, is there)
+        KF_TRY(dev_alloc(p.ozBox, std::max<size_t>(pinv_oz_box_bytes(npl, (int)p.nleaves), 16)));
+        KF_TRY(dev_alloc(p.ozEb, (size_t)(p.nleaves + 128) * 4));
+    }
     KF_CUDA(cudaStreamSynchronize(st));
     dev_free(M);
     p.lat_up = true;
