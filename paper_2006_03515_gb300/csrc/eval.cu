@@ -1174,26 +1174,51 @@ __global__ void __launch_bounds__(P2M_T) k_s2l_x(EvalView E, const int32_t* boxe
     }
 }
 
-// Targets, far part: local expansion of the leaf (y = c_B + r_out r_B s_k, density phi_d)
-// and the W list (y = c_A + r_in r_A s_k, density phi_u). One block per leaf, one thread
-// per target point. Writes far[i] for every point of the leaf.
+// FP32 sum over staged surface points (plain sums of 8 terms, compensated across blocks); PLAIN: no
+// pair closer than 0.5 / (b - a)
+template <bool PLAIN>
+__device__ __forceinline__ Kahan surf_sum(Kahan acc, const float4& xl, const float4* s32, int ns, const KParams& kp) {
+    int e = 0;
+    for (; e + 7 < ns; e += 8) {
+        float part = 0.f;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const float4 v = s32[e + u];
+            const float dx = xl.x - v.x, dy = xl.y - v.y, dz = xl.z - v.z;
+            const float r2 = dx * dx + dy * dy + dz * dz;
+            part = fmaf(PLAIN ? kern_plain_f32(r2, kp) : kern_f32(r2, kp), v.w, part);
+        }
+        acc.add(part);
+    }
+    for (; e < ns; ++e) {
+        const float4 v = s32[e];
+        const float dx = xl.x - v.x, dy = xl.y - v.y, dz = xl.z - v.z;
+        const float r2 = dx * dx + dy * dy + dz * dz;
+        acc.add((PLAIN ? kern_plain_f32(r2, kp) : kern_f32(r2, kp)) * v.w);
+    }
+    return acc;
+}
+
+// Targets, far part: local expansion of the leaf (y = c_B + r_out r_B s_k, density phi_d). One block
+// per leaf, one thread per target point. Writes far[i] for every point of the leaf; the W list adds to
+// it in k_m2p (in one kernel, the few leaves with W lists of up to 148 boxes, two warps each, ran on
+// alone: 2.40 ms for the 51,000 leaves of the two-level grid of 3.2 M cells, 868 of them with W lists;
+// apart 0.31 and 0.41 ms).
 constexpr int L2P_T = 64;
-// SER: some target of a leaf may lie closer than 0.5 / (b - a) to its downward equivalent
-// surface (the W-list sources always take the series-safe form)
+// SER: some target of a leaf may lie closer than 0.5 / (b - a) to its downward equivalent surface
 template <bool MIXED, bool SER, class TD>
-__global__ void __launch_bounds__(L2P_T) k_l2p(EvalView E, const int32_t* leaves, const int32_t* woff,
-                                             const int32_t* witems, const TD* phi_d,
-                                             const TD* phi_u, double* far) {
+__global__ void __launch_bounds__(L2P_T) k_l2p(EvalView E, const int32_t* leaves, const TD* phi_d, double* far) {
     const int B = leaves[blockIdx.x];
     const int S = E.S;
     const int lev = E.level[B];
-    const double* cB = E.centre + 3 * (int64_t)B;
     __shared__ float4 s32[320];
     __shared__ double s64[320][4];
     __shared__ Pair64Tab tab;
     if (!MIXED) p64_load(E, tab);
     const int p0 = E.pstart[B], p1 = E.pend[B];
-    const int nsrc_lists = 1 + (woff[B + 1] - woff[B]);
+    const double* cB = E.centre + 3 * (int64_t)B;
+    const bool local = lev >= 2 && !E.cheb;   // Chebyshev: interpolation in k_l2p_cheb
+    const double rad = E.rf_out * half_width(E, lev);
     for (int t0 = p0; t0 < p1; t0 += L2P_T) {
         const int i = t0 + threadIdx.x;
         const bool act = i < p1;
@@ -1203,67 +1228,93 @@ __global__ void __launch_bounds__(L2P_T) k_l2p(EvalView E, const int32_t* leaves
             for (int k = 0; k < 3; ++k) x64[k] = E.pts[3 * (int64_t)i + k] - cB[k];
         Kahan acc32;
         double acc64 = 0;
-        for (int li = 0; li < nsrc_lists; ++li) {
-            int A;
-            double rad;
-            const TD* dens;
-            int ld = S;
-            if (li == 0) {
-                if (lev < 2 || E.cheb) continue;   // Chebyshev: interpolation in k_l2p_cheb
-                A = B;
-                rad = E.rf_out * half_width(E, lev);
-                dens = phi_d;
-            } else {
-                A = witems[woff[B] + li - 1];
-                rad = E.rf_ueq * half_width(E, E.level[A]);
-                dens = phi_u;
-                ld = E.ldu;
-            }
-            const double* cA = E.centre + 3 * (int64_t)A;
-            const double d[3] = {cA[0] - cB[0], cA[1] - cB[1], cA[2] - cB[2]};
-            for (int s0 = 0; s0 < S; s0 += 320) {
-                const int ns = min(320, S - s0);
-                __syncthreads();
-                for (int e = threadIdx.x; e < ns; e += L2P_T) {
-                    const double* sv = E.surf + 3 * (s0 + e);
-                    double y0 = d[0] + rad * sv[0], y1 = d[1] + rad * sv[1], y2 = d[2] + rad * sv[2];
-                    double ph = (double)dens[(int64_t)A * ld + s0 + e];
-                    if (MIXED) s32[e] = make_float4((float)y0, (float)y1, (float)y2, (float)ph);
-                    else {
-                        s64[e][0] = y0; s64[e][1] = y1; s64[e][2] = y2; s64[e][3] = ph;
-                    }
-                }
-                __syncthreads();
-                if (!act) continue;
-                if (MIXED) {
-                    const bool plain = !SER && li == 0;
-                    int e = 0;
-                    for (; e + 7 < ns; e += 8) {   // plain FP32 sums of 8 terms, compensated across blocks
-                        float part = 0.f;
-#pragma unroll
-                        for (int u = 0; u < 8; ++u) {
-                            const float4 v = s32[e + u];
-                            const float dx = xl.x - v.x, dy = xl.y - v.y, dz = xl.z - v.z;
-                            const float r2 = dx * dx + dy * dy + dz * dz;
-                            part = fmaf(plain ? kern_plain_f32(r2, E.kp) : kern_f32(r2, E.kp), v.w, part);
-                        }
-                        acc32.add(part);
-                    }
-                    for (; e < ns; ++e) {
-                        const float4 v = s32[e];
-                        const float dx = xl.x - v.x, dy = xl.y - v.y, dz = xl.z - v.z;
-                        const float r2 = dx * dx + dy * dy + dz * dz;
-                        acc32.add((plain ? kern_plain_f32(r2, E.kp) : kern_f32(r2, E.kp)) * v.w);
-                    }
-                } else {
-                    for (int e = 0; e < ns; ++e) {
-                        const double dx = x64[0] - s64[e][0], dy = x64[1] - s64[e][1], dz = x64[2] - s64[e][2];
-                        acc64 += p64_pair(dx * dx + dy * dy + dz * dz, E, tab) * s64[e][3];
-                    }
+        for (int s0 = 0; local && s0 < S; s0 += 320) {
+            const int ns = min(320, S - s0);
+            __syncthreads();
+            for (int e = threadIdx.x; e < ns; e += L2P_T) {
+                const double* sv = E.surf + 3 * (s0 + e);
+                const double y0 = rad * sv[0], y1 = rad * sv[1], y2 = rad * sv[2];
+                const double ph = (double)phi_d[(int64_t)B * S + s0 + e];
+                if (MIXED) s32[e] = make_float4((float)y0, (float)y1, (float)y2, (float)ph);
+                else {
+                    s64[e][0] = y0; s64[e][1] = y1; s64[e][2] = y2; s64[e][3] = ph;
                 }
             }
+            __syncthreads();
+            if (!act) continue;
+            if (MIXED) acc32 = surf_sum<!SER>(acc32, xl, s32, ns, E.kp);
+            else
+                for (int e = 0; e < ns; ++e) {
+                    const double dx = x64[0] - s64[e][0], dy = x64[1] - s64[e][1], dz = x64[2] - s64[e][2];
+                    acc64 += p64_pair(dx * dx + dy * dy + dz * dz, E, tab) * s64[e][3];
+                }
         }
         if (act) far[i] = MIXED ? acc32.value() : acc64;
+    }
+}
+
+// The W list at the targets of a leaf that has one (y = c_A + r_in r_A s_k, density phi_u): far += its
+// sum. One block per leaf: eight groups of 64 targets take every eighth box of the list, each staging its
+// own; the groups' sums are added in order.
+constexpr int M2P_G = 8, M2P_T = 64 * M2P_G, M2P_CH = 152;
+template <bool MIXED, class TD>
+__global__ void __launch_bounds__(M2P_T) k_m2p(EvalView E, const int32_t* wleaves, const int32_t* woff,
+                                               const int32_t* witems, const TD* phi_u, double* far) {
+    const int B = wleaves[blockIdx.x];
+    const int S = E.S, g = threadIdx.x >> 6, tl = threadIdx.x & 63;
+    extern __shared__ __align__(16) unsigned char smem_raw[];   // per group M2P_CH sources
+    float4* s32 = reinterpret_cast<float4*>(smem_raw) + g * M2P_CH;
+    double* s64 = reinterpret_cast<double*>(smem_raw) + g * M2P_CH * 4;
+    __shared__ double red[M2P_G][64];
+    __shared__ Pair64Tab tab;
+    if (!MIXED) p64_load(E, tab);
+    __syncthreads();
+    const double* cB = E.centre + 3 * (int64_t)B;
+    const int p0 = E.pstart[B], p1 = E.pend[B], w0 = woff[B], w1 = woff[B + 1];
+    for (int t0 = p0; t0 < p1; t0 += 64) {
+        const int i = t0 + tl;
+        const bool act = i < p1;
+        float4 xl = act ? E.loc[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+        double x64[3] = {0, 0, 0};
+        if (!MIXED && act)
+            for (int k = 0; k < 3; ++k) x64[k] = E.pts[3 * (int64_t)i + k] - cB[k];
+        Kahan acc32;
+        double acc64 = 0;
+        for (int wi = w0 + g; wi < w1; wi += M2P_G) {
+            const int A = witems[wi];
+            const double rad = E.rf_ueq * half_width(E, E.level[A]);
+            const double* cA = E.centre + 3 * (int64_t)A;
+            const double d[3] = {cA[0] - cB[0], cA[1] - cB[1], cA[2] - cB[2]};
+            for (int s0 = 0; s0 < S; s0 += M2P_CH) {
+                const int ns = min(M2P_CH, S - s0);
+                asm volatile("bar.sync %0, 64;" ::"r"(g + 1) : "memory");   // the group's two warps
+                for (int e = tl; e < ns; e += 64) {
+                    const double* sv = E.surf + 3 * (s0 + e);
+                    const double y0 = d[0] + rad * sv[0], y1 = d[1] + rad * sv[1], y2 = d[2] + rad * sv[2];
+                    const double ph = (double)phi_u[(int64_t)A * E.ldu + s0 + e];
+                    if (MIXED) s32[e] = make_float4((float)y0, (float)y1, (float)y2, (float)ph);
+                    else {
+                        s64[4 * e] = y0; s64[4 * e + 1] = y1; s64[4 * e + 2] = y2; s64[4 * e + 3] = ph;
+                    }
+                }
+                asm volatile("bar.sync %0, 64;" ::"r"(g + 1) : "memory");
+                if (!act) continue;
+                if (MIXED) acc32 = surf_sum<false>(acc32, xl, s32, ns, E.kp);
+                else
+                    for (int e = 0; e < ns; ++e) {
+                        const double dx = x64[0] - s64[4 * e], dy = x64[1] - s64[4 * e + 1], dz = x64[2] - s64[4 * e + 2];
+                        acc64 += p64_pair(dx * dx + dy * dy + dz * dz, E, tab) * s64[4 * e + 3];
+                    }
+            }
+        }
+        red[g][tl] = MIXED ? acc32.value() : acc64;
+        __syncthreads();
+        if (g == 0 && act) {
+            double s = 0.0;
+            for (int k = 0; k < M2P_G; ++k) s += red[k][tl];
+            far[i] += s;
+        }
+        __syncthreads();
     }
 }
 
@@ -2139,16 +2190,23 @@ int run_eval(Plan& p, const void* I, void* S_out, int dtype, double C) {
             --nl;   // (counted below)
         } else if (mixed) {
             auto* kl2p = p.far_series ? k_l2p<true, true, float> : k_l2p<true, false, float>;
-            kl2p<<<(unsigned)p.nleaves, L2P_T, 0, st>>>(E, ptr<int32_t>(p.leaves), wo, wi, ptr<float>(p.phid),
-                                                        p.cheb ? ptr<float>(p.cu32) : ptr<float>(p.phiu),
-                                                        ptr<double>(p.far));
+            kl2p<<<(unsigned)p.nleaves, L2P_T, 0, st>>>(E, ptr<int32_t>(p.leaves), ptr<float>(p.phid), ptr<double>(p.far));
         } else {
-            k_l2p<false, true, double><<<(unsigned)p.nleaves, L2P_T, 0, st>>>(
-                E, ptr<int32_t>(p.leaves), wo, wi, ptr<double>(p.phid), p.cheb ? ptr<double>(p.cu) : ptr<double>(p.phiu),
-                ptr<double>(p.far));
+            k_l2p<false, true, double><<<(unsigned)p.nleaves, L2P_T, 0, st>>>(E, ptr<int32_t>(p.leaves),
+                                                                              ptr<double>(p.phid), ptr<double>(p.far));
         }
         KF_LAUNCH();
         ++nl;
+        if (p.n_wleaves > 0) {
+            if (mixed)
+                k_m2p<true, float><<<p.n_wleaves, M2P_T, M2P_G * M2P_CH * 16, st>>>(
+                    E, ptr<int32_t>(p.wleaves), wo, wi, p.cheb ? ptr<float>(p.cu32) : ptr<float>(p.phiu), ptr<double>(p.far));
+            else
+                k_m2p<false, double><<<p.n_wleaves, M2P_T, M2P_G * M2P_CH * 32, st>>>(
+                    E, ptr<int32_t>(p.wleaves), wo, wi, p.cheb ? ptr<double>(p.cu) : ptr<double>(p.phiu), ptr<double>(p.far));
+            KF_LAUNCH();
+            ++nl;
+        }
         if (p.cheb && t.nlevels > 2) {   // (on a lattice the 512-row matrix kernel was slower than this)
             if (mixed)
                 k_l2p_cheb<true, float><<<(unsigned)p.nleaves, L2P_T, 0, st>>>(E, ptr<int32_t>(p.leaves), ptr<float>(p.dd),
