@@ -56,15 +56,37 @@ __device__ __forceinline__ double pair64_min(double x, double hi) {
     return xh > hh && xh < 0x7ff00000 ? hi : x;
 }
 
+// 1 / sqrt(x), x > 0: the approximate reciprocal square root and one third-order step
+__device__ __forceinline__ double rsqrt64(double x) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-(x * y), y, 1.0);
+    return fma(y * e, fma(0.375, e, 0.5), y);
+}
+
+// e^{-x} for x >= 0 (0 above 690)
+__device__ __forceinline__ double exp_neg64(double x, const Pair64Tab& tab) {
+    constexpr double L = 0.69314718055994530942 / kPairTab, MAGIC = 6755399441055744.0;
+    constexpr double c = kPairTab * 1.4426950408889634074, cl = kPairTab * 2.0355273740931033e-17;
+    const double X = pair64_min(x, 691.0);
+    double k = fma(X, c, MAGIC);
+    const int i = __double2loint(k);
+    k -= MAGIC;
+    const double f = fma(-X, cl, fma(-X, c, k));
+    double p = fma(f, L * L * L * L / 24, L * L * L / 6);
+    p = fma(p, f, L * L / 2);
+    p = fma(p, f, L);
+    p *= f;
+    double s = tab.t[i & (kPairTab - 1)];
+    s = __hiloint2double(__double2hiint(s) - ((i >> 8) << 20), __double2loint(s));
+    return __double2hiint(X) > __double2hiint(690.0) ? 0.0 : fma(s, p, s);
+}
+
 // e^{-aR} - e^{-bR} times norm / R^3; r2 > 0
 __device__ __forceinline__ double pair64_kernel(double r2, const Pair64& k, const Pair64Tab& tab) {
     constexpr double L = 0.69314718055994530942 / kPairTab;   // ln2 / 256
     constexpr double MAGIC = 6755399441055744.0;              // 1.5 2^52: x + MAGIC holds rint(x) in its low word
-    double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(r2));
-    double t = r2 * y;
-    const double e = fma(-t, y, 1.0);
-    y = fma(y * e, fma(0.375, e, 0.5), y);
+    const double y = rsqrt64(r2);
     const double R = r2 * y;
     // e^{-aR} = s (1 + p): s = 2^{-ka/256}
     const double Ra = pair64_min(R, k.ra), Rm = pair64_min(R, k.rm);
