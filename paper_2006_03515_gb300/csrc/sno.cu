@@ -59,7 +59,7 @@ struct SnoModel {
     std::vector<int64_t> off;        // offsets: Wl, bl, then per layer Rr, Ri, W, b, then Q1, q1, Q2, q2
     DevBuf theta, grad, adam_m, adam_v, rbf;   // rbf: BF16 copies of Rr, Ri per layer
     DevBuf tabs;                     // float2 twiddle tables
-    int64_t tzf, tyf, tzb, txi, tzi, tzr;   // table offsets (float2 units)
+    int64_t tzf, tyf, tzb, tzi, tzr, tfo, tph;   // table offsets (float2 units)
     // fields (FP32): v[L+1][B][C][np3], z[L][B][C][np3], dz ping-pong [2][B][C][np3], y and dy [B][np3]
     DevBuf v, z, dz, yb, dy, loss;
     // spectra (float2): cz [B][C][n][n][m], cy / gx [B][C][n][2m][m], gy [B][C][n][n][m],
@@ -121,11 +121,12 @@ __device__ __forceinline__ float gelu_d(float x) {
 }
 
 // Twiddle tables: tzf[kz][z] = e^{-i kz z}, tzb = (w/N^3) e^{-i kz z}, tyf[k][y] = e^{-i k y}
-// (k = 0..2m-1 mapped to {0..m-1} U {N-m..N-1}), txi[x][k] = e^{+i k x},
-// tzi[z][kz] = (w/N^3) e^{+i kz z}, tzr[z][kz] = e^{+i kz z} (angles in 2 pi / N units, N the
-// period, grid indices 0..n-1).
-__global__ void k_tables(int n, int N, int m, float2* t, int64_t tzf, int64_t tyf, int64_t tzb, int64_t txi,
-                         int64_t tzi, int64_t tzr) {
+// (k = 0..2m-1 mapped to {0..m-1} U {N-m..N-1}), tzi[z][kz] = (w/N^3) e^{+i kz z},
+// tzr[z][kz] = e^{+i kz z}, tfo[j][k] = (cos, sin)(k (zc - j)) for j < n / 2 and k = 0..m with
+// zc = (n - 1) / 2, tph[k] = (cos, sin)(k zc) (angles in 2 pi / N units, N the period, grid
+// indices 0..n-1).
+__global__ void k_tables(int n, int N, int m, float2* t, int64_t tzf, int64_t tyf, int64_t tzb, int64_t tzi,
+                         int64_t tzr, int64_t tfo, int64_t tph) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const double tw = 6.283185307179586476925286766559 / N;
     const double n3 = (double)N * N * N;
@@ -142,10 +143,14 @@ __global__ void k_tables(int n, int N, int m, float2* t, int64_t tzf, int64_t ty
         double a = tw * kxy(k) * y;
         t[tyf + i] = make_float2((float)cos(a), (float)-sin(a));
     }
-    if (i < n * 2 * m) {
-        int x = i / (2 * m), k = i % (2 * m);
-        double a = tw * kxy(k) * x;
-        t[txi + i] = make_float2((float)cos(a), (float)sin(a));
+    if (i < n / 2 * (m + 1)) {
+        int j = i / (m + 1), k = i % (m + 1);
+        double a = tw * k * (0.5 * (n - 1) - j);
+        t[tfo + i] = make_float2((float)cos(a), (float)sin(a));
+    }
+    if (i <= m) {
+        double a = tw * i * (0.5 * (n - 1));
+        t[tph + i] = make_float2((float)cos(a), (float)sin(a));
     }
     if (i < n * m) {
         int z = i / m, kz = i % m;
@@ -153,63 +158,6 @@ __global__ void k_tables(int n, int N, int m, float2* t, int64_t tzf, int64_t ty
         double w = (kz == 0 ? 1.0 : 2.0) / n3;
         t[tzi + i] = make_float2((float)(w * cos(a)), (float)(w * sin(a)));
         t[tzr + i] = make_float2((float)cos(a), (float)sin(a));
-    }
-}
-
-// Plane DFT: out[p][j][i] = sum_q T[j][q] in[p][q][i] (complex), p < P, j < Lout, i < inner.
-// A block takes PB planes (or one plane and a chunk of ICH columns), stages them in shared
-// memory and computes every output of those columns; T is read through the L1 cache.
-__global__ void __launch_bounds__(256) k_plane(const float2* __restrict__ in, float2* __restrict__ out,
-                                               const float2* __restrict__ T, int64_t P, int Lin, int Lout, int inner,
-                                               int PB, int ICH, int nch) {
-    extern __shared__ float2 psh[];   // [Lin][ncol] inputs, then T [Lout][Lin]
-    const int64_t pb = blockIdx.x / nch;
-    const int ch = (int)(blockIdx.x % nch);
-    const int64_t p0 = pb * PB;
-    const int np = (int)min((int64_t)PB, P - p0);
-    const int i0 = ch * ICH;
-    const int W = min(ICH, inner - i0);
-    const int ncol = np * W;
-    for (int e = threadIdx.x; e < Lin * ncol; e += blockDim.x) {
-        const int q = e / ncol, col = e % ncol;
-        const int pl = col / W, w = col % W;
-        psh[q * ncol + col] = in[((p0 + pl) * Lin + q) * (int64_t)inner + i0 + w];
-    }
-    float2* Ts = psh + Lin * ncol;
-    for (int e = threadIdx.x; e < Lout * Lin; e += blockDim.x) Ts[e] = T[e];
-    __syncthreads();
-    // each thread: 8 consecutive outputs j0..j0+7 of two columns (col, col + ncol/2); the
-    // columns' inputs are read once per q and T[j][q] is uniform across the warp
-    const int njb = (Lout + 7) / 8, nch2 = (ncol + 1) / 2;
-    for (int e = threadIdx.x; e < njb * nch2; e += blockDim.x) {
-        const int jb = e / nch2, c0 = e % nch2;
-        const int c1 = c0 + nch2 < ncol ? c0 + nch2 : c0;
-        const int j0 = 8 * jb;
-        const int nj = min(8, Lout - j0);
-        const float2* t0 = Ts + j0 * Lin;
-        float re[2][8], im[2][8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) re[0][u] = im[0][u] = re[1][u] = im[1][u] = 0.f;
-        for (int q = 0; q < Lin; ++q) {
-            const float2 x0 = psh[q * ncol + c0], x1 = psh[q * ncol + c1];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const float2 a = t0[min(u, nj - 1) * Lin + q];
-                re[0][u] = fmaf(a.x, x0.x, fmaf(-a.y, x0.y, re[0][u]));
-                im[0][u] = fmaf(a.x, x0.y, fmaf(a.y, x0.x, im[0][u]));
-                re[1][u] = fmaf(a.x, x1.x, fmaf(-a.y, x1.y, re[1][u]));
-                im[1][u] = fmaf(a.x, x1.y, fmaf(a.y, x1.x, im[1][u]));
-            }
-        }
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            if (h == 1 && c1 == c0) break;
-            const int col = h ? c1 : c0;
-            const int pl = col / W, w = col % W;
-#pragma unroll
-            for (int u = 0; u < 8; ++u)
-                if (u < nj) out[((p0 + pl) * Lout + j0 + u) * (int64_t)inner + i0 + w] = make_float2(re[h][u], im[h][u]);
-        }
     }
 }
 
@@ -223,85 +171,193 @@ __device__ __forceinline__ void sno_cp16(void* dst, const void* src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
 }
 __device__ __forceinline__ void sno_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void sno_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 __device__ __forceinline__ void sno_wait_prev() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
 
-// Plane DFT, persistent and double-buffered: the same contraction as k_plane over tiles of
-// PB planes (or one plane and a chunk of ICH columns); each block walks its tiles with the
-// next tile's inputs copied asynchronously into the second buffer while it computes the
-// current one, so the global loads overlap the arithmetic. T stays in shared memory.
-__global__ void __launch_bounds__(256) k_plane2(const float2* __restrict__ in, float2* __restrict__ out,
-                                                const float2* __restrict__ T, int64_t P, int Lin, int Lout,
-                                                int inner, int PB, int ICH, int nch, int64_t ntiles) {
-    extern __shared__ float2 psh[];   // T [Lout][Lin], then two buffers [Lin][PB * ICH]
-    float2* Ts = psh;
-    const int cmax = PB * min(ICH, inner);
-    float2* const buf0 = psh + Lout * Lin;   // buffer k at buf0 + k Lin cmax
-    for (int e = threadIdx.x; e < Lout * Lin; e += blockDim.x) Ts[e] = T[e];
-    auto shape = [&](int64_t t, int64_t& p0, int& np, int& i0, int& W) {
-        const int64_t pb = t / nch;
-        p0 = pb * PB;
-        np = (int)min((int64_t)PB, P - p0);
-        i0 = (int)(t % nch) * ICH;
-        W = min(ICH, inner - i0);
-    };
-    auto issue = [&](int64_t t, float2* dst) {   // a thread per column, down the Lin rows
-        int64_t p0;
-        int np, i0, W;
-        shape(t, p0, np, i0, W);
-        const int ncol = np * W;
-        for (int col = threadIdx.x; col < ncol; col += blockDim.x) {
-            const int pl = col / W, w = col - pl * W;
-            const float2* src = in + (p0 + pl) * Lin * (int64_t)inner + i0 + w;
-            for (int q = 0; q < Lin; ++q) sno_cp8(dst + q * ncol + col, src + (int64_t)q * inner);
+// Plane DFTs along x and y, folded: in[p][q][i] -> out[p][j][i] with p < P planes and i < inner
+// columns. About the grid's centre zc = (n - 1) / 2 the points q and n - 1 - q lie at -t and
+// +t, so a frequency pair +-k needs only P_k = sum_t cos(k t) s_t and Q_k = sum_t sin(k t) d_t
+// of the sums and differences s, d of the two points (forward: F(+-k) = e^{-+i k zc} (P_k -+ i Q_k)),
+// and a point pair only U_t = sum_k cos(k t) a_k and V_t = sum_k sin(k t) b_k of those of the two
+// frequencies (inverse: f(+-t) = U_t +- i V_t): a quarter of the dense form's FMAs. What is
+// left is bound by memory: persistent blocks copy the next tile of columns (whole planes
+// where they are short, else a chunk of columns of one plane) in 16-byte pieces, the way it
+// lies in memory, while they compute the current one.
+// One GB300, 32 fields of 64^3 at width 32 and 12 modes: 16 passes 3.55 -> 1.66 ms
+// (the dense form read its tiles in 8-byte pieces); the largest, 554 MB, 419 -> 176 us = 3.1 TB/s.
+struct FoldTile {
+    int64_t P, ntiles;
+    int L, inner, PB, W, nch, ps;   // rows in, columns in all, planes and columns a tile, chunks, plane stride
+};
+__device__ __forceinline__ void fold_shape(const FoldTile& f, int64_t t, int64_t& p0, int& np, int& i0, int& w) {
+    const int64_t pb = t / f.nch;
+    p0 = pb * f.PB;
+    np = (int)min((int64_t)f.PB, f.P - p0);
+    i0 = (int)(t - pb * f.nch) * f.W;
+    w = min(f.W, f.inner - i0);
+}
+// copies tile t to dst[pl][q][w] (rows of f.W, planes of f.ps elements)
+__device__ __forceinline__ void fold_issue(const FoldTile& f, int64_t t, const float2* __restrict__ in, float2* dst) {
+    int64_t p0;
+    int np, i0, w;
+    fold_shape(f, t, p0, np, i0, w);
+    if (f.nch == 1) {   // whole planes: contiguous, an even number of elements (L is even)
+        const int half = f.L * f.inner / 2;
+        for (int pl = 0; pl < np; ++pl) {
+            const float2* src = in + (p0 + pl) * f.L * (int64_t)f.inner;
+            for (int r = threadIdx.x; r < half; r += blockDim.x) sno_cp16(dst + pl * f.ps + 2 * r, src + 2 * r);
         }
-    };
+        return;
+    }
+    const float2* src = in + p0 * f.L * (int64_t)f.inner + i0;
+    const int lane = threadIdx.x & 31;
+    if (f.inner % 2 == 0) {   // (f.W is even, so is the last chunk's width)
+        for (int q = threadIdx.x >> 5; q < f.L; q += blockDim.x >> 5)
+            for (int r = lane; r < w / 2; r += 32) sno_cp16(dst + q * f.W + 2 * r, src + (int64_t)q * f.inner + 2 * r);
+    } else {
+        for (int q = threadIdx.x >> 5; q < f.L; q += blockDim.x >> 5)
+            for (int r = lane; r < w; r += 32) sno_cp8(dst + q * f.W + r, src + (int64_t)q * f.inner + r);
+    }
+}
+
+constexpr int FF_T = 128;   // threads of the forward kernel
+constexpr int FV_T = 256;   // and of the inverse
+constexpr int FV_J = 8;     // point pairs a thread of the inverse
+
+// n points to 2m frequencies; a thread takes one column and KB frequencies (of 0..m)
+template <int KB>
+__global__ void __launch_bounds__(FF_T) k_fold_fwd(const float2* __restrict__ in, float2* __restrict__ out,
+                                                   const float2* __restrict__ tfo, const float2* __restrict__ tph,
+                                                   int m, int nkb, FoldTile f) {
+    constexpr int KP = (KB + 1) & ~1;   // (a table row is read in 16-byte pieces)
+    extern __shared__ __align__(16) float2 psh[];
+    const int n = f.L, nh = n / 2, bufn = f.PB * f.ps;
+    float2* T = psh;                    // [nkb][n / 2][KP], zero past m
+    float2* buf = T + nkb * nh * KP;    // two tiles
+    for (int e = threadIdx.x; e < nkb * nh * KP; e += FF_T) {
+        const int u = e % KP, j = (e / KP) % nh, k = (e / (KP * nh)) * KB + u;
+        T[e] = u < KB && k <= m ? tfo[j * (m + 1) + k] : make_float2(0.f, 0.f);
+    }
     int64_t t = blockIdx.x;
-    if (t < ntiles) issue(t, buf0);
+    if (t < f.ntiles) fold_issue(f, t, in, buf);
     sno_commit();
-    for (int it = 0; t < ntiles; t += gridDim.x, ++it) {
-        const int64_t tn = t + gridDim.x;
-        if (tn < ntiles) issue(tn, buf0 + (size_t)((it + 1) & 1) * Lin * cmax);
+    for (int it = 0; t < f.ntiles; t += gridDim.x, ++it) {
+        sno_wait_all();
+        __syncthreads();   // the tile is there, and the other buffer has been read
+        if (t + gridDim.x < f.ntiles) fold_issue(f, t + gridDim.x, in, buf + ((it + 1) & 1) * bufn);
         sno_commit();
-        sno_wait_prev();
-        __syncthreads();
-        const float2* X = buf0 + (size_t)(it & 1) * Lin * cmax;
         int64_t p0;
-        int np, i0, W;
-        shape(t, p0, np, i0, W);
-        const int ncol = np * W;
-        // each thread: 8 consecutive outputs j0..j0+7 of two columns (col, col + ncol/2)
-        const int njb = (Lout + 7) / 8, nch2 = (ncol + 1) / 2;
-        for (int e = threadIdx.x; e < njb * nch2; e += blockDim.x) {
-            const int jb = e / nch2, c0 = e % nch2;
-            const int c1 = c0 + nch2 < ncol ? c0 + nch2 : c0;
-            const int j0 = 8 * jb;
-            const int nj = min(8, Lout - j0);
-            const float2* t0 = Ts + j0 * Lin;
-            float re[2][8], im[2][8];
+        int np, i0, w;
+        fold_shape(f, t, p0, np, i0, w);
+        const int ncol = np * w;
+        for (int e = threadIdx.x; e < nkb * ncol; e += FF_T) {
+            const int kb = e / ncol, col = e - kb * ncol, pl = col / w, i = col - pl * w;
+            const float2* lo = buf + (it & 1) * bufn + pl * f.ps + i;
+            const float2* hi = lo + (n - 1) * f.W;
+            const float4* tk = reinterpret_cast<const float4*>(T + kb * nh * KP);
+            float pr[KP], pi[KP], qr[KP], qi[KP];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) re[0][u] = im[0][u] = re[1][u] = im[1][u] = 0.f;
-            for (int q = 0; q < Lin; ++q) {
-                const float2 x0 = X[q * ncol + c0], x1 = X[q * ncol + c1];
+            for (int u = 0; u < KP; ++u) pr[u] = pi[u] = qr[u] = qi[u] = 0.f;
+            for (int j = 0; j < nh; ++j, lo += f.W, hi -= f.W, tk += KP / 2) {
+                const float2 x0 = *lo, x1 = *hi;
+                const float sr = x1.x + x0.x, si = x1.y + x0.y, dr = x1.x - x0.x, di = x1.y - x0.y;
 #pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const float2 a = t0[min(u, nj - 1) * Lin + q];
-                    re[0][u] = fmaf(a.x, x0.x, fmaf(-a.y, x0.y, re[0][u]));
-                    im[0][u] = fmaf(a.x, x0.y, fmaf(a.y, x0.x, im[0][u]));
-                    re[1][u] = fmaf(a.x, x1.x, fmaf(-a.y, x1.y, re[1][u]));
-                    im[1][u] = fmaf(a.x, x1.y, fmaf(a.y, x1.x, im[1][u]));
+                for (int u = 0; u < KP; u += 2) {
+                    const float4 c = tk[u / 2];
+                    pr[u] = fmaf(c.x, sr, pr[u]);
+                    pi[u] = fmaf(c.x, si, pi[u]);
+                    qr[u] = fmaf(c.y, dr, qr[u]);
+                    qi[u] = fmaf(c.y, di, qi[u]);
+                    if (u + 1 < KB) {
+                        pr[u + 1] = fmaf(c.z, sr, pr[u + 1]);
+                        pi[u + 1] = fmaf(c.z, si, pi[u + 1]);
+                        qr[u + 1] = fmaf(c.w, dr, qr[u + 1]);
+                        qi[u + 1] = fmaf(c.w, di, qi[u + 1]);
+                    }
                 }
             }
+            float2* o = out + (p0 + pl) * 2 * m * (int64_t)f.inner + i0 + i;
 #pragma unroll
-            for (int hh = 0; hh < 2; ++hh) {
-                if (hh == 1 && c1 == c0) break;
-                const int col = hh ? c1 : c0;
-                const int pl = col / W, w = col % W;
-#pragma unroll
-                for (int u = 0; u < 8; ++u)
-                    if (u < nj) out[((p0 + pl) * Lout + j0 + u) * (int64_t)inner + i0 + w] = make_float2(re[hh][u], im[hh][u]);
+            for (int u = 0; u < KB; ++u) {
+                const int k = kb * KB + u;
+                if (k > m) break;
+                const float2 ph = __ldg(tph + k);
+                const float ar = pr[u] + qi[u], ai = pi[u] - qr[u], br = pr[u] - qi[u], bi = pi[u] + qr[u];
+                if (k < m) o[(int64_t)k * f.inner] = make_float2(fmaf(ar, ph.x, ai * ph.y), fmaf(ai, ph.x, -ar * ph.y));
+                if (k > 0)
+                    o[(int64_t)(2 * m - k) * f.inner] = make_float2(fmaf(br, ph.x, -bi * ph.y), fmaf(bi, ph.x, br * ph.y));
             }
         }
-        __syncthreads();   // the buffer is refilled two tiles later
+    }
+}
+
+// 2m frequencies to n points; the tile's frequency pairs are folded once, then a thread takes
+// one column and FV_J point pairs
+__global__ void __launch_bounds__(FV_T) k_fold_inv(const float2* __restrict__ in, float2* __restrict__ out,
+                                                   const float2* __restrict__ tfo, const float2* __restrict__ tph,
+                                                   int m, int n, int njb, FoldTile f) {
+    extern __shared__ __align__(16) float2 psh[];
+    const int m1 = m + 1, nh = n / 2, bufn = f.PB * f.ps, NJ = njb * FV_J;
+    float2* T = psh;                                       // [m + 1][NJ], zero past n / 2
+    float4* F = reinterpret_cast<float4*>(T + m1 * NJ);    // [m + 1][PB W]: a, b
+    float2* buf = reinterpret_cast<float2*>(F + m1 * f.PB * f.W);
+    for (int e = threadIdx.x; e < m1 * NJ; e += FV_T) {
+        const int k = e / NJ, j = e - k * NJ;
+        T[e] = j < nh ? tfo[j * m1 + k] : make_float2(0.f, 0.f);
+    }
+    int64_t t = blockIdx.x;
+    if (t < f.ntiles) fold_issue(f, t, in, buf);
+    sno_commit();
+    for (int it = 0; t < f.ntiles; t += gridDim.x, ++it) {
+        sno_wait_all();
+        __syncthreads();   // the tile is there, the other buffer and F have been read
+        if (t + gridDim.x < f.ntiles) fold_issue(f, t + gridDim.x, in, buf + ((it + 1) & 1) * bufn);
+        sno_commit();
+        int64_t p0;
+        int np, i0, w;
+        fold_shape(f, t, p0, np, i0, w);
+        const int ncol = np * w;
+        for (int e = threadIdx.x; e < m1 * ncol; e += FV_T) {
+            const int k = e / ncol, col = e - k * ncol, pl = col / w, i = col - pl * w;
+            const float2* x = buf + (it & 1) * bufn + pl * f.ps + i;
+            const float2 g = k < m ? x[k * f.W] : make_float2(0.f, 0.f);
+            const float2 h = k > 0 ? x[(2 * m - k) * f.W] : make_float2(0.f, 0.f);
+            const float2 ph = __ldg(tph + k);
+            const float gr = fmaf(g.x, ph.x, -g.y * ph.y), gi = fmaf(g.x, ph.y, g.y * ph.x);
+            const float hr = fmaf(h.x, ph.x, h.y * ph.y), hi = fmaf(h.y, ph.x, -h.x * ph.y);
+            F[e] = make_float4(gr + hr, gi + hi, gr - hr, gi - hi);
+        }
+        __syncthreads();
+        for (int e = threadIdx.x; e < njb * ncol; e += FV_T) {
+            const int jb = e / ncol, col = e - jb * ncol, pl = col / w, i = col - pl * w;
+            float ur[FV_J], ui[FV_J], vr[FV_J], vi[FV_J];
+#pragma unroll
+            for (int u = 0; u < FV_J; ++u) ur[u] = ui[u] = vr[u] = vi[u] = 0.f;
+            for (int k = 0; k < m1; ++k) {
+                const float4 x = F[k * ncol + col];
+                const float4* tk = reinterpret_cast<const float4*>(T + k * NJ + jb * FV_J);
+#pragma unroll
+                for (int u = 0; u < FV_J; u += 2) {
+                    const float4 c = tk[u / 2];
+                    ur[u] = fmaf(c.x, x.x, ur[u]);
+                    ui[u] = fmaf(c.x, x.y, ui[u]);
+                    vr[u] = fmaf(c.y, x.z, vr[u]);
+                    vi[u] = fmaf(c.y, x.w, vi[u]);
+                    ur[u + 1] = fmaf(c.z, x.x, ur[u + 1]);
+                    ui[u + 1] = fmaf(c.z, x.y, ui[u + 1]);
+                    vr[u + 1] = fmaf(c.w, x.z, vr[u + 1]);
+                    vi[u + 1] = fmaf(c.w, x.w, vi[u + 1]);
+                }
+            }
+            float2* o = out + (p0 + pl) * n * (int64_t)f.inner + i0 + i;
+#pragma unroll
+            for (int u = 0; u < FV_J; ++u) {
+                const int j = jb * FV_J + u;
+                if (j >= nh) break;
+                o[(int64_t)j * f.inner] = make_float2(ur[u] + vi[u], ui[u] - vr[u]);
+                o[(int64_t)(n - 1 - j) * f.inner] = make_float2(ur[u] - vi[u], ui[u] + vr[u]);
+            }
+        }
     }
 }
 
@@ -510,125 +566,6 @@ __global__ void __launch_bounds__(ZR_T) k_lift_z(const float* __restrict__ u, co
         }
         __syncthreads();
         zfwd_rows(vs, tf, C, n, m, cz + (b * C * n2 + xy) * m, n2 * m);
-    }
-}
-
-// forward, layer output side: z = Re(Tzi gy) + W v + b, v_next = GELU(z) (or z for the last
-// layer); optional: z stored (training), next layer's cz = Tzf v_next, projection y.
-// Main loop: a thread takes channels o0..o0+3 at the two points zp and zp + n/2.
-__global__ void __launch_bounds__(ZR_T) k_zinv_point(const float2* __restrict__ gy, const float* __restrict__ v,
-                                                     const float* __restrict__ W, const float* __restrict__ bias,
-                                                     const float2* __restrict__ Tzi, const float2* __restrict__ Tzf,
-                                                     float* __restrict__ zout, float* __restrict__ vnext,
-                                                     float2* __restrict__ cznext, const float* __restrict__ Q1,
-                                                     const float* __restrict__ q1, const float* __restrict__ Q2,
-                                                     const float* __restrict__ q2, float* __restrict__ y, int B, int C,
-                                                     int n, int m, int P, int act) {
-    extern __shared__ float zsh[];
-    const int ns = n + 1, C1 = C + 1;
-    float* vs = zsh;                     // [C][n + 1]
-    float* vo = vs + C * ns;             // [C][n + 1]
-    float* Ws = vo + C * ns;             // [C][C + 1]
-    float* bs = Ws + C * C1;             // [C]
-    float* Qs = bs + C;                  // [P][C + 1] (projection)
-    float* ypart = Qs + (y ? P * C1 : 0);            // [4][n]
-    float* pq = ypart + (y ? 4 * n : 0);             // q1, Q2 [2][P]
-    size_t fo = (size_t)(pq + (y ? 2 * P : 0) - zsh);
-    fo = (fo + 1) & ~(size_t)1;
-    float2* gs = reinterpret_cast<float2*>(zsh + fo);   // [C][m]
-    float2* ti = gs + C * m;                            // [n][m + 1]
-    float2* tf = ti + n * (m + 1);                      // [m][n + 1]
-    for (int e = threadIdx.x; e < C * C; e += blockDim.x) Ws[(e / C) * C1 + e % C] = W[e];
-    for (int e = threadIdx.x; e < C; e += blockDim.x) bs[e] = bias[e];
-    for (int e = threadIdx.x; e < n * m; e += blockDim.x) ti[(e / m) * (m + 1) + e % m] = Tzi[e];
-    if (cznext)
-        for (int e = threadIdx.x; e < m * n; e += blockDim.x) tf[(e / n) * ns + e % n] = Tzf[e];
-    if (y) {
-        for (int e = threadIdx.x; e < P * C; e += blockDim.x) Qs[(e / C) * C1 + e % C] = Q1[e];
-        for (int e = threadIdx.x; e < P; e += blockDim.x) {
-            pq[e] = q1[e];
-            pq[P + e] = Q2[e];
-        }
-    }
-    const int64_t n2 = (int64_t)n * n, rows = (int64_t)B * n2;
-    const int zb = (n + 1) / 2, obn = (C + 3) / 4;
-    for (int64_t r = (int64_t)blockIdx.x * ZR_RG; r < min(rows, (int64_t)(blockIdx.x + 1) * ZR_RG); ++r) {
-        const int64_t b = r / n2, xy = r % n2;
-        __syncthreads();
-        for (int e = threadIdx.x; e < C * n; e += blockDim.x) {
-            const int c = e / n, zz = e % n;
-            vs[c * ns + zz] = v[((b * C + c) * n2 + xy) * n + zz];
-        }
-        for (int e = threadIdx.x; e < C * m; e += blockDim.x) {
-            const int o = e / m, kz = e % m;
-            gs[e] = gy[((b * C + o) * n2 + xy) * m + kz];
-        }
-        __syncthreads();
-        for (int e = threadIdx.x; e < obn * zb; e += blockDim.x) {
-            const int z0 = e % zb, o0 = 4 * (e / zb);
-            const int z1 = z0 + zb < n ? z0 + zb : z0;
-            int oc[4];
-            float a0[4], a1[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                oc[u] = min(o0 + u, C - 1);
-                a0[u] = a1[u] = bs[oc[u]];
-            }
-            const float2* t0 = ti + z0 * (m + 1);
-            const float2* t1 = ti + z1 * (m + 1);
-            for (int kz = 0; kz < m; ++kz) {
-                const float2 ta = t0[kz], tb = t1[kz];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const float2 g = gs[oc[u] * m + kz];
-                    a0[u] = fmaf(ta.x, g.x, fmaf(-ta.y, g.y, a0[u]));
-                    a1[u] = fmaf(tb.x, g.x, fmaf(-tb.y, g.y, a1[u]));
-                }
-            }
-            for (int c = 0; c < C; ++c) {
-                const float x0 = vs[c * ns + z0], x1 = vs[c * ns + z1];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const float w = Ws[oc[u] * C1 + c];
-                    a0[u] = fmaf(w, x0, a0[u]);
-                    a1[u] = fmaf(w, x1, a1[u]);
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                if (o0 + u >= C) break;
-                const int o = o0 + u;
-                const int64_t g0 = ((b * C + o) * n2 + xy) * n;
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    if (h == 1 && z1 == z0) break;
-                    const int zz = h ? z1 : z0;
-                    const float av = h ? a1[u] : a0[u];
-                    if (zout) zout[g0 + zz] = av;
-                    const float vv = act ? gelu_f(av) : av;
-                    vo[o * ns + zz] = vv;
-                    vnext[g0 + zz] = vv;
-                }
-            }
-        }
-        __syncthreads();
-        if (cznext) zfwd_rows(vo, tf, C, n, m, cznext + (b * C * n2 + xy) * m, n2 * m);
-        if (y) {   // y = q2 + sum_p Q2[p] GELU(q1[p] + Q1[p] . v); thread = (point, quarter of p)
-            for (int e = threadIdx.x; e < 4 * n; e += blockDim.x) {
-                const int zz = e % n, part = e / n;
-                float acc = 0.f;
-                for (int p = part; p < P; p += 4) {
-                    const float* qr = Qs + p * C1;
-                    float a = pq[p];
-                    for (int c = 0; c < C; ++c) a = fmaf(qr[c], vo[c * ns + zz], a);
-                    acc = fmaf(pq[P + p], gelu_f(a), acc);
-                }
-                ypart[part * n + zz] = acc;
-            }
-            __syncthreads();
-            for (int e = threadIdx.x; e < n; e += blockDim.x)
-                y[b * n2 * n + xy * n + e] = q2[0] + ((ypart[e] + ypart[n + e]) + (ypart[2 * n + e] + ypart[3 * n + e]));
-        }
     }
 }
 
@@ -1433,39 +1370,56 @@ __global__ void k_to_bf16(const float* a, __nv_bfloat16* b, int64_t n) {
 // ---- passes ---------------------------------------------------------------------------------
 static float* fld(const DevBuf& b, int64_t i, int64_t per) { return ptr<float>(b) + i * per; }
 
-// plane DFT launch: columns per block about 64 (several planes when inner is short)
-static int plane(SnoModel& M, const float2* in, float2* out, int64_t tab, int64_t P, int Lin, int Lout, int inner) {
-    // tiles of about 2 x 256 / ceil(Lout / 8) columns: one (8 outputs x 2 columns) item per thread
-    const int njb = (Lout + 7) / 8;
-    // about 2 x 256 / njb columns (one item per thread), at most 48 KB of inputs per buffer
-    const int target = std::max(8, std::min(512 / njb, (48 << 10) / (8 * Lin)));
-    int PB = 1, ICH = inner;
-    if (inner >= target) {
-        const int nchunk = (inner + target - 1) / target;
-        ICH = (inner + nchunk - 1) / nchunk;
-    } else {
-        PB = std::max(1, target / inner);
+// tiles of about `cols` columns for the folded plane transforms
+static FoldTile fold_tiles(int64_t P, int L, int inner, int cols) {
+    FoldTile f;
+    f.P = P;
+    f.L = L;
+    f.inner = inner;
+    f.PB = 1;
+    f.W = inner;
+    f.ps = L * inner;
+    if (inner > cols) {
+        const int nchunk = (inner + cols - 1) / cols;
+        f.W = ((inner + nchunk - 1) / nchunk + 1) & ~1;
+        f.ps = L * f.W;
+    } else {   // the planes' stride continues the columns' banks, and keeps the 16-byte copies aligned
+        f.PB = (int)std::min<int64_t>(std::max(1, cols / inner), P);
+        f.ps += (((inner + 1) & ~1) - L * inner % 16 + 16) % 16;
     }
-    const int nch = (inner + ICH - 1) / ICH;
-    const int64_t ntiles = ((P + PB - 1) / PB) * nch;
-    const size_t smem = ((size_t)2 * Lin * PB * std::min(ICH, inner) + (size_t)Lout * Lin) * sizeof(float2);
-    if (smem > 160 * 1024) {   // (larger shapes than the model's: the single-shot kernel)
-        int PB1 = 1, ICH1 = inner;
-        if (inner >= 128) ICH1 = 128;
-        else PB1 = std::max(1, 128 / inner);
-        const int nch1 = (inner + ICH1 - 1) / ICH1;
-        const int64_t nb = ((P + PB1 - 1) / PB1) * nch1;
-        const size_t smem1 = ((size_t)Lin * PB1 * std::min(ICH1, inner) + (size_t)Lout * Lin) * sizeof(float2);
-        k_plane<<<(unsigned)nb, 256, smem1, M.st>>>(in, out, ptr<float2>(M.tabs) + tab, P, Lin, Lout, inner, PB1, ICH1,
-                                                    nch1);
-        KF_LAUNCH();
-        return KIFMM_OK;
-    }
+    f.nch = (inner + f.W - 1) / f.W;
+    f.ntiles = ((P + f.PB - 1) / f.PB) * f.nch;
+    return f;
+}
+
+// x and y transforms of [P][n][inner] to [P][2m][inner]: about one item a thread, at most 72 KB of
+// tiles (three blocks an SM at n = 64)
+static int plane_fwd(SnoModel& M, const float2* in, float2* out, int64_t P, int inner) {
+    const int nkb = (M.m + 8) / 8, kb = std::max(4, (M.m + nkb) / nkb), kp = (kb + 1) & ~1;
+    const FoldTile f = fold_tiles(P, M.n, inner, std::max(2, std::min(FF_T / nkb, (72 << 10) / (16 * M.n))) & ~1);
+    const size_t smem = ((size_t)2 * f.PB * f.ps + (size_t)nkb * (M.n / 2) * kp) * sizeof(float2);
+    auto* k = kb == 4 ? k_fold_fwd<4> : kb == 5 ? k_fold_fwd<5> : kb == 6 ? k_fold_fwd<6> : kb == 7 ? k_fold_fwd<7>
+                                                                                         : k_fold_fwd<8>;
     int per_sm = 1;
-    KF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_plane2, 256, smem));
-    const int64_t grid = std::min<int64_t>(ntiles, (int64_t)std::max(1, per_sm) * M.num_sms);
-    k_plane2<<<(unsigned)grid, 256, smem, M.st>>>(in, out, ptr<float2>(M.tabs) + tab, P, Lin, Lout, inner, PB, ICH,
-                                                  nch, ntiles);
+    KF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, FF_T, smem));
+    const int64_t grid = std::min<int64_t>(f.ntiles, (int64_t)std::max(1, per_sm) * M.num_sms);
+    const float2* T = ptr<float2>(M.tabs);
+    k<<<(unsigned)grid, FF_T, smem, M.st>>>(in, out, T + M.tfo, T + M.tph, M.m, nkb, f);
+    KF_LAUNCH();
+    return KIFMM_OK;
+}
+// and of [P][2m][inner] to [P][n][inner]
+static int plane_inv(SnoModel& M, const float2* in, float2* out, int64_t P, int inner) {
+    const int njb = (M.n / 2 + FV_J - 1) / FV_J;
+    const FoldTile f = fold_tiles(P, 2 * M.m, inner,
+                                  std::max(2, std::min(FV_T / njb, (80 << 10) / (48 * M.m + 16))) & ~1);
+    const size_t smem = ((size_t)2 * f.PB * f.ps + (size_t)(M.m + 1) * njb * FV_J) * sizeof(float2) +
+                        (size_t)(M.m + 1) * f.PB * f.W * sizeof(float4);
+    int per_sm = 1;
+    KF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fold_inv, FV_T, smem));
+    const int64_t grid = std::min<int64_t>(f.ntiles, (int64_t)std::max(1, per_sm) * M.num_sms);
+    const float2* T = ptr<float2>(M.tabs);
+    k_fold_inv<<<(unsigned)grid, FV_T, smem, M.st>>>(in, out, T + M.tfo, T + M.tph, M.m, M.n, njb, f);
     KF_LAUNCH();
     return KIFMM_OK;
 }
@@ -1518,8 +1472,8 @@ static int forward(SnoModel& M, const float* u, float* y, int B, bool train) {
         k_lift_u<<<(unsigned)((rows + LU - 1) / LU), 256, (size_t)LU * n * 4 + (size_t)m * n * 8, st>>>(
             u, T + M.tzf, ptr<float2>(M.cz), rows, n, m);
         KF_LAUNCH();
-        KF_TRY(plane(M, ptr<float2>(M.cz), ptr<float2>(M.cy), M.tyf, (int64_t)B * n, n, M2, m));     // y
-        KF_TRY(plane(M, ptr<float2>(M.cy), ptr<float2>(M.Vst), M.tyf, B, n, M2, M2 * m));           // x: U
+        KF_TRY(plane_fwd(M, ptr<float2>(M.cz), ptr<float2>(M.cy), (int64_t)B * n, m));     // y
+        KF_TRY(plane_fwd(M, ptr<float2>(M.cy), ptr<float2>(M.Vst), B, M2 * m));           // x: U
         float2* A = ptr<float2>(M.m0ab);
         float2* Bc = A + (int64_t)C * M.K;
         const unsigned np = nbs((int64_t)C * M.K, 256);
@@ -1542,12 +1496,12 @@ static int forward(SnoModel& M, const float* u, float* y, int B, bool train) {
     for (int l = 0; l < M.L; ++l) {
         if (!(inf && l == 0)) {
             float2* V = ptr<float2>(M.Vst) + (train ? (int64_t)l * BC * M.K : 0);
-            KF_TRY(plane(M, ptr<float2>(M.cz), ptr<float2>(M.cy), M.tyf, BC * n, n, M2, m));            // y
-            KF_TRY(plane(M, ptr<float2>(M.cy), V, M.tyf, BC, n, M2, M2 * m));                            // x
+            KF_TRY(plane_fwd(M, ptr<float2>(M.cz), ptr<float2>(M.cy), BC * n, m));            // y
+            KF_TRY(plane_fwd(M, ptr<float2>(M.cy), V, BC, M2 * m));                            // x
             KF_TRY(mix(M, l, V, ptr<float2>(M.g), B, 0));
         }
-        KF_TRY(plane(M, ptr<float2>(M.g), ptr<float2>(M.gx), M.txi, BC, M2, n, M2 * m));             // x^-1
-        KF_TRY(plane(M, ptr<float2>(M.gx), ptr<float2>(M.gy), M.txi, BC * n, M2, n, m));             // y^-1
+        KF_TRY(plane_inv(M, ptr<float2>(M.g), ptr<float2>(M.gx), BC, M2 * m));             // x^-1
+        KF_TRY(plane_inv(M, ptr<float2>(M.gx), ptr<float2>(M.gy), BC * n, m));             // y^-1
         const bool last = l == M.L - 1;
         if (inf) {
             const size_t sm = last ? M.zi_smem_y : M.zi_smem;
@@ -1598,15 +1552,15 @@ static int loss_grad(SnoModel& M, const float* u, const float* t, int B, double*
     KF_LAUNCH();
     for (int l = L - 1; l >= 0; --l) {
         // spectral adjoint of layer l: dG = Tyf Tyf Tzb dz_l (cz holds Tzb dz_l), dR, dV = R^H dG
-        KF_TRY(plane(M, ptr<float2>(M.cz), ptr<float2>(M.cy), M.tyf, BC * n, n, M2, m));
-        KF_TRY(plane(M, ptr<float2>(M.cy), ptr<float2>(M.g), M.tyf, BC, n, M2, M2 * m));
+        KF_TRY(plane_fwd(M, ptr<float2>(M.cz), ptr<float2>(M.cy), BC * n, m));
+        KF_TRY(plane_fwd(M, ptr<float2>(M.cy), ptr<float2>(M.g), BC, M2 * m));
         const unsigned nb = nbs(M.K, M.mix_mb);
         k_mix_grad<<<nb, 256, M.mixg_smem, st>>>(ptr<float2>(M.g), ptr<float2>(M.Vst) + (int64_t)l * BC * M.K,
                                                  gr + M.off[o_rr(l)], gr + M.off[o_ri(l)], B, C, M.K, M.mix_mb);
         KF_LAUNCH();
         KF_TRY(mix(M, l, ptr<float2>(M.g), ptr<float2>(M.ga), B, 1));
-        KF_TRY(plane(M, ptr<float2>(M.ga), ptr<float2>(M.gx), M.txi, BC, M2, n, M2 * m));
-        KF_TRY(plane(M, ptr<float2>(M.gx), ptr<float2>(M.gy), M.txi, BC * n, M2, n, m));
+        KF_TRY(plane_inv(M, ptr<float2>(M.ga), ptr<float2>(M.gx), BC, M2 * m));
+        KF_TRY(plane_inv(M, ptr<float2>(M.gx), ptr<float2>(M.gy), BC * n, m));
         if (l > 0) {
             k_zinv_point_bwd<<<zr_blocks(M, B), ZR_T, M.zr_smem_f, st>>>(
                 ptr<float2>(M.gy), dzA, th + M.off[o_w(l)], T + M.tzr, fld(M.z, l - 1, per), fld(M.v, l - 1, per),
@@ -1967,12 +1921,12 @@ int sno_create(sno_model_t* out, int n, int width, int modes, int layers, int pr
         }
         const int lim = optin;
         cudaFuncSetAttribute(k_lift_z, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-        cudaFuncSetAttribute(k_zinv_point, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
         cudaFuncSetAttribute(k_zrow_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
         cudaFuncSetAttribute(k_zinv_point_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
         cudaFuncSetAttribute(k_proj_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-        cudaFuncSetAttribute(k_plane, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-        cudaFuncSetAttribute(k_plane2, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+        for (auto* k : {k_fold_fwd<4>, k_fold_fwd<5>, k_fold_fwd<6>, k_fold_fwd<7>, k_fold_fwd<8>})
+            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+        cudaFuncSetAttribute(k_fold_inv, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
         cudaFuncSetAttribute(k_zrow_inf<32, 64, 12>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
         cudaFuncSetAttribute(k_zrow_inf<0, 0, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
         if (M.zi_smem_y > (size_t)lim) M.zi_smem = M.zi_smem_y = 0;
@@ -2003,13 +1957,14 @@ int sno_create(sno_model_t* out, int n, int width, int modes, int layers, int pr
     M.tzf = 0;
     M.tyf = M.tzf + (int64_t)modes * n;
     M.tzb = M.tyf + (int64_t)2 * modes * n;
-    M.txi = M.tzb + (int64_t)modes * n;
-    M.tzi = M.txi + (int64_t)n * 2 * modes;
+    M.tzi = M.tzb + (int64_t)modes * n;
     M.tzr = M.tzi + (int64_t)n * modes;
-    if ((rc = dev_alloc(M.tabs, (M.tzr + (int64_t)n * modes) * sizeof(float2)))) return fail(rc);
+    M.tfo = M.tzr + (int64_t)n * modes;
+    M.tph = M.tfo + (int64_t)n / 2 * (modes + 1);
+    if ((rc = dev_alloc(M.tabs, (M.tph + modes + 1) * sizeof(float2)))) return fail(rc);
     M.period = n;
     k_tables<<<nbs(2 * modes * n, 128), 128, 0, M.st>>>(n, n, modes, ptr<float2>(M.tabs), M.tzf, M.tyf, M.tzb,
-                                                          M.txi, M.tzi, M.tzr);
+                                                          M.tzi, M.tzr, M.tfo, M.tph);
     if (cudaGetLastError() != cudaSuccess) return fail(KIFMM_ERR_CUDA);
     if ((rc = dev_alloc(M.v, (size_t)(layers + 1) * per * 4))) return fail(rc);
     if ((rc = dev_alloc(M.z, (size_t)layers * per * 4))) return fail(rc);
@@ -2051,7 +2006,7 @@ int sno_set_period(sno_model_t h, int period) {
     }
     M.period = period;
     k_tables<<<nbs(2 * M.m * M.n, 128), 128, 0, M.st>>>(M.n, period, M.m, ptr<float2>(M.tabs), M.tzf, M.tyf, M.tzb,
-                                                          M.txi, M.tzi, M.tzr);
+                                                          M.tzi, M.tzr, M.tfo, M.tph);
     KF_LAUNCH();
     KF_CUDA(cudaStreamSynchronize(M.st));
     return KIFMM_OK;
