@@ -63,3 +63,26 @@ def test_forward_and_gradient_match_oracle(n, period, C, m, L, P, B):
         scale = np.linalg.norm(g[off:off + k]) + 1e-6 * ref
         assert abs(float(g @ d) - fd) <= 2e-3 * scale, (name, float(g @ d), fd, scale)
         off += k
+
+
+@pytest.mark.parametrize("n, r_in, r_out", [(12, 0.5, 1.0), (12, 1.0, 2.5), (20, 2.0, 5.0), (24, 3.0, 7.0),
+                                            (28, 4.0, 8.0), (36, 2.0, 4.0)])
+@pytest.mark.parametrize("offset", [0, 1])
+def test_near_part_matches_oracle(n, r_in, r_out, offset):
+    """The near part alone (all parameters zero) for every kind of halo, grids that are no multiple of
+    the kernel's tile, and a field that starts off a 16-byte boundary."""
+    import torch
+    from oracle import kernel as K
+    a, b, h = 5.25, 300.0, 1.0 / n
+    M = kifmm.SNO(n, 4, 1, 1, 1, max_batch=2)
+    M.set_params(np.zeros(M.num_params(), np.float32))
+    M.set_near_field(a, b, h, r_in, r_out)
+    u = np.random.Generator(np.random.PCG64(n)).standard_normal((2, n, n, n)).astype(np.float32)
+    buf = torch.zeros(u.size + 1, device="cuda")
+    du = buf[offset:offset + u.size].copy_(torch.as_tensor(u.ravel())).view(2, -1)
+    y = M.forward(du).cpu().numpy()
+    M.close()
+    sigma = K.self_sigma(h, a, b, "cell_exact")
+    for i in range(2):
+        ref = O.near_field(u[i].astype(np.float64), a, b, h, sigma, r_in, r_out).ravel()
+        assert np.abs(y[i] - ref).max() <= 1e-5 * np.abs(ref).max()
