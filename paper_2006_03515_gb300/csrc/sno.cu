@@ -59,7 +59,7 @@ struct SnoModel {
     std::vector<int64_t> off;        // offsets: Wl, bl, then per layer Rr, Ri, W, b, then Q1, q1, Q2, q2
     DevBuf theta, grad, adam_m, adam_v, rbf;   // rbf: BF16 copies of Rr, Ri per layer
     DevBuf tabs;                     // float2 twiddle tables
-    int64_t tzf, tyf, tzb, tzi, tzr, tfo, tph;   // table offsets (float2 units)
+    int64_t tzf, tyf, tzb, tzr, tfo, tph;   // table offsets (float2 units)
     // fields (FP32): v[L+1][B][C][np3], z[L][B][C][np3], dz ping-pong [2][B][C][np3], y and dy [B][np3]
     DevBuf v, z, dz, yb, dy, loss;
     // spectra (float2): cz [B][C][n][n][m], cy / gx [B][C][n][2m][m], gy [B][C][n][n][m],
@@ -68,8 +68,7 @@ struct SnoModel {
     DevBuf m0ab;                     // inference, layer 0: A = R Wl and Bc = (R bl) O, [2][C][K] complex
     DevBuf jt, jref, jorig, jerr;    // photo_solve judge: targets, reference values, caller indices, error
     int mix_mb = 1;                  // modes per block of the mixing kernels
-    size_t zr_smem_f = 0, zr_smem_b = 0, zr_smem_p = 0, mix_smem = 0, mixg_smem = 0, zf_smem = 0;
-    size_t zi_smem = 0, zi_smem_y = 0;   // k_zrow_inf (0: the shape does not suit it)
+    size_t zr_smem_f = 0, zr_smem_b = 0, mix_smem = 0, mixg_smem = 0;
     int num_sms = 1;
     int64_t steps = 0;
     int period = 0;                  // N of the transforms (>= n)
@@ -121,12 +120,11 @@ __device__ __forceinline__ float gelu_d(float x) {
 }
 
 // Twiddle tables: tzf[kz][z] = e^{-i kz z}, tzb = (w/N^3) e^{-i kz z}, tyf[k][y] = e^{-i k y}
-// (k = 0..2m-1 mapped to {0..m-1} U {N-m..N-1}), tzi[z][kz] = (w/N^3) e^{+i kz z},
-// tzr[z][kz] = e^{+i kz z}, tfo[j][k] = (cos, sin)(k (zc - j)) for j < n / 2 and k = 0..m with
-// zc = (n - 1) / 2, tph[k] = (cos, sin)(k zc) (angles in 2 pi / N units, N the period, grid
-// indices 0..n-1).
-__global__ void k_tables(int n, int N, int m, float2* t, int64_t tzf, int64_t tyf, int64_t tzb, int64_t tzi,
-                         int64_t tzr, int64_t tfo, int64_t tph) {
+// (k = 0..2m-1 mapped to {0..m-1} U {N-m..N-1}), tzr[z][kz] = e^{+i kz z},
+// tfo[j][k] = (cos, sin)(k (zc - j)) for j < n / 2 and k = 0..m with zc = (n - 1) / 2,
+// tph[k] = (cos, sin)(k zc) (angles in 2 pi / N units, N the period, grid indices 0..n-1).
+__global__ void k_tables(int n, int N, int m, float2* t, int64_t tzf, int64_t tyf, int64_t tzb, int64_t tzr,
+                         int64_t tfo, int64_t tph) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const double tw = 6.283185307179586476925286766559 / N;
     const double n3 = (double)N * N * N;
@@ -155,8 +153,6 @@ __global__ void k_tables(int n, int N, int m, float2* t, int64_t tzf, int64_t ty
     if (i < n * m) {
         int z = i / m, kz = i % m;
         double a = tw * kz * z;
-        double w = (kz == 0 ? 1.0 : 2.0) / n3;
-        t[tzi + i] = make_float2((float)(w * cos(a)), (float)(w * sin(a)));
         t[tzr + i] = make_float2((float)cos(a), (float)sin(a));
     }
 }
@@ -225,6 +221,18 @@ __device__ __forceinline__ void fold_issue(const FoldTile& f, int64_t t, const f
     }
 }
 
+// Factor of column i (kz = i mod m): the z rows' transforms are taken about their centre as well, and
+// their phase e^{+i kz zc} belongs to the x transforms, where the spectra are smallest. zscale = 0: the
+// rows' transforms are not centred, factor 1; else zscale, twice that for kz > 0 where it is not 1
+// (1 / N^3 of the inverse transform and the conjugate half of the spectrum).
+__device__ __forceinline__ float2 fold_zphase(const float2* __restrict__ tph, int m, int i, float zscale) {
+    if (zscale == 0.f) return make_float2(1.f, 0.f);
+    const int kz = i % m;
+    const float w = zscale != 1.f && kz > 0 ? 2.f * zscale : zscale;
+    const float2 ph = __ldg(tph + kz);
+    return make_float2(w * ph.x, w * ph.y);
+}
+
 constexpr int FF_T = 128;   // threads of the forward kernel
 constexpr int FV_T = 256;   // and of the inverse
 constexpr int FV_J = 8;     // point pairs a thread of the inverse
@@ -233,7 +241,7 @@ constexpr int FV_J = 8;     // point pairs a thread of the inverse
 template <int KB>
 __global__ void __launch_bounds__(FF_T) k_fold_fwd(const float2* __restrict__ in, float2* __restrict__ out,
                                                    const float2* __restrict__ tfo, const float2* __restrict__ tph,
-                                                   int m, int nkb, FoldTile f) {
+                                                   int m, int nkb, float zscale, FoldTile f) {
     constexpr int KP = (KB + 1) & ~1;   // (a table row is read in 16-byte pieces)
     extern __shared__ __align__(16) float2 psh[];
     const int n = f.L, nh = n / 2, bufn = f.PB * f.ps;
@@ -282,15 +290,18 @@ __global__ void __launch_bounds__(FF_T) k_fold_fwd(const float2* __restrict__ in
                 }
             }
             float2* o = out + (p0 + pl) * 2 * m * (int64_t)f.inner + i0 + i;
+            const float2 z = fold_zphase(tph, m, i0 + i, zscale);   // (conjugated: this is the forward direction)
 #pragma unroll
             for (int u = 0; u < KB; ++u) {
                 const int k = kb * KB + u;
                 if (k > m) break;
                 const float2 ph = __ldg(tph + k);
                 const float ar = pr[u] + qi[u], ai = pi[u] - qr[u], br = pr[u] - qi[u], bi = pi[u] + qr[u];
-                if (k < m) o[(int64_t)k * f.inner] = make_float2(fmaf(ar, ph.x, ai * ph.y), fmaf(ai, ph.x, -ar * ph.y));
+                const float2 a = make_float2(fmaf(ar, ph.x, ai * ph.y), fmaf(ai, ph.x, -ar * ph.y));
+                const float2 b = make_float2(fmaf(br, ph.x, -bi * ph.y), fmaf(bi, ph.x, br * ph.y));
+                if (k < m) o[(int64_t)k * f.inner] = make_float2(fmaf(a.x, z.x, a.y * z.y), fmaf(a.y, z.x, -a.x * z.y));
                 if (k > 0)
-                    o[(int64_t)(2 * m - k) * f.inner] = make_float2(fmaf(br, ph.x, -bi * ph.y), fmaf(bi, ph.x, br * ph.y));
+                    o[(int64_t)(2 * m - k) * f.inner] = make_float2(fmaf(b.x, z.x, b.y * z.y), fmaf(b.y, z.x, -b.x * z.y));
             }
         }
     }
@@ -300,7 +311,7 @@ __global__ void __launch_bounds__(FF_T) k_fold_fwd(const float2* __restrict__ in
 // one column and FV_J point pairs
 __global__ void __launch_bounds__(FV_T) k_fold_inv(const float2* __restrict__ in, float2* __restrict__ out,
                                                    const float2* __restrict__ tfo, const float2* __restrict__ tph,
-                                                   int m, int n, int njb, FoldTile f) {
+                                                   int m, int n, int njb, float zscale, FoldTile f) {
     extern __shared__ __align__(16) float2 psh[];
     const int m1 = m + 1, nh = n / 2, bufn = f.PB * f.ps, NJ = njb * FV_J;
     float2* T = psh;                                       // [m + 1][NJ], zero past n / 2
@@ -330,7 +341,10 @@ __global__ void __launch_bounds__(FV_T) k_fold_inv(const float2* __restrict__ in
             const float2 ph = __ldg(tph + k);
             const float gr = fmaf(g.x, ph.x, -g.y * ph.y), gi = fmaf(g.x, ph.y, g.y * ph.x);
             const float hr = fmaf(h.x, ph.x, h.y * ph.y), hi = fmaf(h.y, ph.x, -h.x * ph.y);
-            F[e] = make_float4(gr + hr, gi + hi, gr - hr, gi - hi);
+            const float2 z = fold_zphase(tph, m, i0 + i, zscale);
+            const float ar = gr + hr, ai = gi + hi, br = gr - hr, bi = gi - hi;
+            F[e] = make_float4(fmaf(ar, z.x, -ai * z.y), fmaf(ar, z.y, ai * z.x), fmaf(br, z.x, -bi * z.y),
+                               fmaf(br, z.y, bi * z.x));
         }
         __syncthreads();
         for (int e = threadIdx.x; e < njb * ncol; e += FV_T) {
@@ -370,28 +384,44 @@ __global__ void __launch_bounds__(FV_T) k_fold_inv(const float2* __restrict__ in
 // spectrum is V0[c][k] = Wl[c] U[k] + bl[c] O[k] (U the truncated transform of u, O that of
 // the field of ones, separable: O = Sx[kx] Sy[ky] Sz[kz] with S the sums of the tables' rows)
 // and the layer's mix G[o][k] = sum_c R[k][o][c] V0[c][k] = A[o][k] U[k] + Bc[o][k].
-// cu[b][x][y][kz] = sum_z Tzf[kz][z] u[b][x][y][z]; a block stages LU rows and the table
-constexpr int LU = 16;
-__global__ void __launch_bounds__(256) k_lift_u(const float* __restrict__ u, const float2* __restrict__ Tzf,
+// cu[b][x][y][kz] = sum_z e^{-i kz (z - zc)} u[b][x][y][z], folded as in k_fold_fwd; a block stages the
+// sums and differences of LU rows, a thread takes 4 rows and 2 modes
+constexpr int LU = 32;
+__global__ void __launch_bounds__(256) k_lift_u(const float* __restrict__ u, const float2* __restrict__ tfo,
                                                 float2* __restrict__ cu, int64_t rows, int n, int m) {
-    extern __shared__ __align__(16) float lsh[];
-    float* us = lsh;                                            // [LU][n]
-    float2* tf = reinterpret_cast<float2*>(lsh + LU * n);       // [m][n]
-    for (int e = threadIdx.x; e < m * n; e += blockDim.x) tf[e] = Tzf[e];
+    extern __shared__ __align__(16) float2 lsh[];
+    const int nh = n / 2, ns = nh + 1, mh = (m + 1) / 2;
+    float2* sd = lsh;               // [LU][n / 2 + 1]
+    float2* tf = sd + LU * ns;      // [n / 2][m + 1]
+    for (int e = threadIdx.x; e < nh * (m + 1); e += blockDim.x) tf[e] = tfo[e];
     const int64_t r0 = (int64_t)blockIdx.x * LU;
     const int nr = (int)min((int64_t)LU, rows - r0);
-    for (int e = threadIdx.x; e < nr * n; e += blockDim.x) us[e] = u[r0 * n + e];
+    for (int e = threadIdx.x; e < nr * nh; e += blockDim.x) {
+        const int rq = e / nh, j = e - rq * nh;
+        const float lo = u[(r0 + rq) * n + j], hi = u[(r0 + rq) * n + n - 1 - j];
+        sd[rq * ns + j] = make_float2(hi + lo, hi - lo);
+    }
     __syncthreads();
-    for (int e = threadIdx.x; e < nr * m; e += blockDim.x) {
-        const int kz = e % m, rq = e / m;
-        float re = 0.f, im = 0.f;
-        for (int zz = 0; zz < n; ++zz) {
-            const float x = us[rq * n + zz];
-            const float2 t = tf[kz * n + zz];
-            re = fmaf(t.x, x, re);
-            im = fmaf(t.y, x, im);
+    for (int e = threadIdx.x; e < ((nr + 3) / 4) * mh; e += blockDim.x) {
+        const int rb = e / mh, k0 = e - rb * mh, k1 = min(k0 + mh, m - 1);
+        float re[4][2] = {}, im[4][2] = {};
+        for (int j = 0; j < nh; ++j) {
+            const float2 t0 = tf[j * (m + 1) + k0], t1 = tf[j * (m + 1) + k1];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float2 x = sd[min(4 * rb + q, nr - 1) * ns + j];
+                re[q][0] = fmaf(t0.x, x.x, re[q][0]);
+                im[q][0] = fmaf(-t0.y, x.y, im[q][0]);
+                re[q][1] = fmaf(t1.x, x.x, re[q][1]);
+                im[q][1] = fmaf(-t1.y, x.y, im[q][1]);
+            }
         }
-        cu[(r0 + rq) * m + kz] = make_float2(re, im);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            if (4 * rb + q >= nr) break;
+            cu[(r0 + 4 * rb + q) * m + k0] = make_float2(re[q][0], im[q][0]);
+            if (k0 + mh < m) cu[(r0 + 4 * rb + q) * m + k0 + mh] = make_float2(re[q][1], im[q][1]);
+        }
     }
 }
 // A[o][k] = sum_c R[k][o][c] Wl[c], Bc[o][k] = (sum_c R[k][o][c] bl[c]) O[k]
@@ -574,455 +604,288 @@ __global__ void __launch_bounds__(ZR_T) k_lift_z(const float* __restrict__ u, co
     }
 }
 
-// Forward, layer output side, inference (no z kept): persistent blocks over pairs of row
-// groups (b, x, y); the next pair's v rows and gy spectra are copied asynchronously into the
-// second buffer while the current pair is computed. Phase A: a thread takes a 4-channel x
-// 4-point tile of z = Re(Tzi gy) + W v + b (tables laid out [kz][z] so that the point
-// dimension is read as float4 without bank conflicts); the tiles then overwrite v with
-// v_next (GELU unless the last layer) in shared memory and in global memory. Phase B: the
-// next layer's cz = Tzf v_next, a thread per (row, channel, 3 modes), or the projection y
-// (4 projection rows x 4 points per thread). Needs the width and n multiples of 4 and at
-// most blockDim phase-A tiles per pass.
-constexpr int FI = 2;   // row groups per pass
-template <int CT, int NT, int MT>
-__global__ void __launch_bounds__(ZR_T, 3) k_zrow_inf(const float2* __restrict__ gy, const float* __restrict__ v,
-                                                      const float* __restrict__ W, const float* __restrict__ bias,
-                                                      const float2* __restrict__ Tzi, const float2* __restrict__ Tzf,
-                                                      float* __restrict__ vnext, float2* __restrict__ cznext,
-                                                      const float* __restrict__ Q1, const float* __restrict__ q1,
-                                                      const float* __restrict__ Q2, const float* __restrict__ q2,
-                                                      float* __restrict__ y, int B, int C_, int n_, int m_, int P, int act,
-                                                      const float* __restrict__ u0, const float* __restrict__ Wl,
-                                                      const float* __restrict__ bl) {
-    // (CT, NT, MT > 0: the width, grid and mode count fixed at compile time, so that the index
-    // arithmetic below reduces to shifts and multiplications)
-    const int C = CT ? CT : C_, n = NT ? NT : n_, m = MT ? MT : m_;
+// Forward, layer output side: persistent blocks over R row groups (b, x, y) at a time,
+// z = Re(sum_kz g e^{i kz (z - zc)}) + W v + b with v_next = GELU(z) (or z for the last layer), then the
+// next layer's cz = sum_z e^{-i kz (z - zc)} v_next or the projection y; z itself is stored when zout is
+// given (training). Layer 0 of the inference takes W v0 + b = (W Wl) u + (W bl + b) from u.
+// The transforms are folded about the row's centre zc = (n - 1) / 2 as in k_fold_fwd (half the FMAs; the
+// phases e^{+-i kz zc} and the weights are in the spectra). A thread computes 8 channels x 4 point pairs:
+// the pairs' shared cosine and sine sums become the two points' values in the same 64 registers, 16 FMAs a
+// 16-byte shared load in W v, and their sums and differences go to shared memory ready for the next
+// transform (4 channels x 3 modes a thread, lanes 8 x 4 so that a warp reads few distinct words). Three
+// blocks an SM cover each other's loads: bound by FP32 issue (FMAs and GELU's erf).
+// One GB300, 32 fields of 64^3 at width 32 and 12 modes: layers 1 and 2 2.28 -> 1.25 ms each,
+// the last with the projection 2.27 -> 1.92 ms, layer 0 0.87 ms; the four launches 6.83 -> 5.3 ms.
+constexpr int ZF_T = 128;
+struct ZRowDims {
+    int nh, nhp, nzb, nob, CP, CG, nz4, TS, PP, R;   // (see zrow_dims)
+    size_t smem;
+};
+static ZRowDims zrow_dims(int n, int C, int m, int P, bool proj) {
+    ZRowDims d;
+    d.nh = n / 2;
+    d.nhp = (d.nh + 3) & ~3;       // point pairs, in blocks of 4
+    d.nzb = d.nhp / 4;
+    d.nob = (C + 7) / 8;           // channel blocks
+    d.CP = 8 * d.nob;
+    d.CG = d.CP + 2;               // row of a mode's spectra (2-way conflicts in the transposing copy)
+    d.nz4 = n + 4;
+    d.TS = d.nhp + 4;              // row of the cosine and sine tables
+    d.PP = (P + 7) & ~7;
+    d.R = ZF_T / (d.nob * d.nzb);  // one tile a thread (n <= 128 and C <= 64: at least one row)
+    size_t f = (size_t)d.R * C * d.nz4 + (size_t)C * d.CP + 2 * d.CP + 2 * (size_t)m * d.TS +
+               2 * (size_t)d.R * m * d.CG;
+    f = (f + 3) & ~(size_t)3;      // (the projection's rows are read in 16-byte pieces)
+    if (proj) f += (size_t)C * d.PP + 2 * d.PP + (size_t)d.R * (d.PP / 8) * n;
+    d.smem = f * 4;
+    return d;
+}
+__device__ __forceinline__ float4 rev4(float4 a) { return make_float4(a.w, a.z, a.y, a.x); }
+template <bool PROJ>
+__global__ void __launch_bounds__(ZF_T, 3) k_zrow(const float2* __restrict__ gy, const float* __restrict__ v,
+                                                  const float* __restrict__ W, const float* __restrict__ bias,
+                                                  const float2* __restrict__ tfo, float* __restrict__ zout,
+                                                  float* __restrict__ vnext, float2* __restrict__ cznext,
+                                                  const float* __restrict__ Q1, const float* __restrict__ q1,
+                                                  const float* __restrict__ Q2, const float* __restrict__ q2,
+                                                  float* __restrict__ y, const float* __restrict__ u0,
+                                                  const float* __restrict__ Wl, const float* __restrict__ bl, int rows,
+                                                  int C, int n, int m, int P, ZRowDims d) {
     extern __shared__ __align__(16) float zsh[];
-    const int nz4 = n + 4, C4 = C + 4, npb = (P + 3) / 4;
-    float* vb = zsh;                                   // [2][FI][C][n + 4]
-    float* Ws = vb + 2 * FI * C * nz4;                 // [C][C + 4]
-    float* bs = Ws + C * C4;                           // [C]
-    float* Qs = bs + C;                                // [P][C + 4] (projection)
-    float* pq = Qs + (y ? P * C4 : 0);                 // q1, Q2 [2][P]
-    float* ys = pq + (y ? 2 * P : 0);                  // [FI][npb][n]
-    size_t fo = (size_t)(ys + (y ? FI * npb * n : 0) - zsh);
-    fo = (fo + 3) & ~(size_t)3;
-    float2* gb = reinterpret_cast<float2*>(zsh + fo);  // [2][FI][C][m]
-    float2* tf = gb + 2 * FI * C * m;                  // [m][n]
-    float* tiR = reinterpret_cast<float*>(tf + m * n); // [m][n]: Re, Im of Tzi[z][kz] at [kz][z]
-    float* tiI = tiR + m * n;
-    for (int e = threadIdx.x; e < C * C; e += blockDim.x) Ws[(e / C) * C4 + e % C] = W[e];
-    for (int e = threadIdx.x; e < C; e += blockDim.x) bs[e] = bias[e];
-    if (u0) {   // layer 0 from u: W v0 + b = (W Wl) u + (W bl + b), in Ws[o][0] and bs[o]
-        __syncthreads();
-        for (int o = threadIdx.x; o < C; o += blockDim.x) {
-            float w1 = 0.f, w0 = bs[o];
+    float* vs = zsh;                                              // [R][C][n + 4]
+    float* Ws = vs + d.R * C * d.nz4;                             // [C][CP], transposed
+    float* bs = Ws + C * d.CP;                                    // [CP] bias, [CP] W Wl
+    float* tc = bs + 2 * d.CP;                                    // [m][TS] cosines, then sines
+    float* tn = tc + m * d.TS;
+    float2* gs = reinterpret_cast<float2*>(tn + m * d.TS);        // [R][m][CG]
+    float* Qs = zsh + (((d.R * C * d.nz4 + C * d.CP + 2 * d.CP + 2 * m * d.TS + 2 * d.R * m * d.CG) + 3) & ~3);
+    float* pq = Qs + C * d.PP;                                    // [C][PP] Q1 transposed; q1, Q2
+    float* ys = pq + 2 * d.PP;                                    // [R][PP / 8][n]
+    const int tid = threadIdx.x, n4 = n / 4, n2 = n * n;
+    for (int e = tid; e < C * d.CP; e += ZF_T) {
+        const int c = e / d.CP, o = e - c * d.CP;
+        Ws[e] = o < C ? W[o * C + c] : 0.f;
+    }
+    for (int o = tid; o < d.CP; o += ZF_T) {
+        float w0 = o < C ? bias[o] : 0.f, w1 = 0.f;
+        if (u0 && o < C)
             for (int c = 0; c < C; ++c) {
-                w1 = fmaf(Ws[o * C4 + c], Wl[c], w1);
-                w0 = fmaf(Ws[o * C4 + c], bl[c], w0);
+                w1 = fmaf(W[o * C + c], Wl[c], w1);
+                w0 = fmaf(W[o * C + c], bl[c], w0);
             }
-            Ws[o * C4 + C] = w1;   // (the row's padding column)
-            bs[o] = w0;
+        bs[o] = w0;
+        bs[d.CP + o] = w1;
+    }
+    for (int e = tid; e < m * d.nhp; e += ZF_T) {   // (the last block's pairs past n / 2 are mirrored ones)
+        const int k = e / d.nhp, j = e - k * d.nhp;
+        const float2 t = tfo[(j < d.nh ? j : n - 1 - j) * (m + 1) + k];
+        tc[k * d.TS + j] = t.x;
+        tn[k * d.TS + j] = j < d.nh ? t.y : -t.y;
+    }
+    if (PROJ) {
+        for (int e = tid; e < C * d.PP; e += ZF_T) {
+            const int c = e / d.PP, p = e - c * d.PP;
+            Qs[e] = p < P ? Q1[p * C + c] : 0.f;
+        }
+        for (int p = tid; p < d.PP; p += ZF_T) {
+            pq[p] = p < P ? q1[p] : 0.f;
+            pq[d.PP + p] = p < P ? Q2[p] : 0.f;
         }
     }
-    for (int e = threadIdx.x; e < n * m; e += blockDim.x) {
-        const float2 t = Tzi[e];
-        tiR[(e % m) * n + e / m] = t.x;
-        tiI[(e % m) * n + e / m] = t.y;
-    }
-    if (cznext)
-        for (int e = threadIdx.x; e < m * n; e += blockDim.x) tf[e] = Tzf[e];
-    if (y) {
-        for (int e = threadIdx.x; e < P * C; e += blockDim.x) Qs[(e / C) * C4 + e % C] = Q1[e];
-        for (int e = threadIdx.x; e < P; e += blockDim.x) {
-            pq[e] = q1[e];
-            pq[P + e] = Q2[e];
-        }
-    }
-    const int64_t n2 = (int64_t)n * n, rows = (int64_t)B * n2;
-    const int64_t ngroups = (rows + FI - 1) / FI;
-    const int n4 = n / 4, ncb = C / 4;
-    const int64_t cstride = n2 * n;   // between channels of v (and of gy, times m / n)
-    auto issue = [&](int64_t g, int buf) {
-        const int64_t r0 = g * FI;
-        const int nr = (int)min((int64_t)FI, rows - r0);
-        for (int rg = 0; rg < nr; ++rg) {
-            const int64_t r = r0 + rg, b = r / n2, xy = r - b * n2;
-            if (u0) {   // layer 0: the u row, in channel 0's place
-                for (int z = threadIdx.x; z < n; z += blockDim.x)   // (a caller's field may lie anywhere)
-                    vb[((buf * FI + rg) * C) * nz4 + z] = u0[r * n + z];
-            } else {
-                const float* src = v + b * C * cstride + xy * n;
-                for (int e = threadIdx.x; e < C * n4; e += blockDim.x) {
-                    const int c = e / n4, q4 = e - c * n4;
-                    sno_cp16(vb + ((buf * FI + rg) * C + c) * nz4 + 4 * q4, src + c * cstride + 4 * q4);
-                }
-            }
-            const float2* gsrc = gy + (b * C * n2 + xy) * m;
-            for (int e = threadIdx.x; e < C * m; e += blockDim.x) {
-                const int o = e / m, kz = e - o * m;
-                sno_cp8(gb + ((buf * FI + rg) * C + o) * m + kz, gsrc + o * n2 * m + kz);
-            }
-        }
-    };
-    int64_t g = blockIdx.x;
-    if (g < ngroups) issue(g, 0);
-    sno_commit();
-    for (int it = 0; g < ngroups; g += gridDim.x, ++it) {
-        const int64_t gn = g + gridDim.x;
-        if (gn < ngroups) issue(gn, (it + 1) & 1);
-        sno_commit();
-        sno_wait_prev();
-        __syncthreads();
-        const int cur = it & 1;
-        const int64_t r0 = g * FI;
-        const int nr = (int)min((int64_t)FI, rows - r0);
-        float* vs = vb + cur * FI * C * nz4;
-        const float2* gs = gb + cur * FI * C * m;
-        // phase A: one 4 x 4 tile per thread
-        const int nitems = nr * ncb * n4;
-        const int e = threadIdx.x;
-        const int zb = e % n4, cb = (e / n4) % ncb, rg = e / (n4 * ncb);
-        const int z0 = 4 * zb, o0 = 4 * cb;
-        float acc[4][4];
-        if (e < nitems) {
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-#pragma unroll
-                for (int i = 0; i < 4; ++i) acc[j][i] = bs[o0 + j];
-            const float2* gr = gs + (rg * C + o0) * m;
-            for (int kz = 0; kz < m; ++kz) {
-                const float4 ra = *reinterpret_cast<const float4*>(tiR + kz * n + z0);
-                const float4 ia = *reinterpret_cast<const float4*>(tiI + kz * n + z0);
-                const float tr[4] = {ra.x, ra.y, ra.z, ra.w}, tim[4] = {ia.x, ia.y, ia.z, ia.w};
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const float2 gg = gr[j * m + kz];
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) acc[j][i] = fmaf(tr[i], gg.x, fmaf(-tim[i], gg.y, acc[j][i]));
-                }
-            }
-            const float* vr = vs + rg * C * nz4 + z0;
+    const bool aligned = (reinterpret_cast<uintptr_t>(u0) & 15) == 0;   // (a caller's field may lie anywhere)
+    // lanes of the copies: 16-byte pieces of a row and modes of a spectrum, in powers of two
+    const int lv = 32 - __clz(n4 - 1), lm = m > 1 ? 32 - __clz(m - 1) : 0;
+    const int zb = tid % d.nzb, ob = (tid / d.nzb) % d.nob, rg = tid / (d.nzb * d.nob);
+    const int z0 = 4 * zb, z1 = n - 4 - z0, o0 = 8 * ob;
+    for (int r0 = blockIdx.x * d.R; r0 < rows; r0 += gridDim.x * d.R) {
+        const int nr = min(d.R, rows - r0);
+        __syncthreads();   // the previous rows have been read
+        for (int rr = 0; rr < nr; ++rr) {
+            const int b = (r0 + rr) / n2, xy = (r0 + rr) - b * n2;
+            const int q = tid & ((1 << lv) - 1);
             if (u0) {
-                const float4 x = *reinterpret_cast<const float4*>(vr);
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const float w1 = Ws[(o0 + j) * C4 + C];
-                    acc[j][0] = fmaf(w1, x.x, acc[j][0]);
-                    acc[j][1] = fmaf(w1, x.y, acc[j][1]);
-                    acc[j][2] = fmaf(w1, x.z, acc[j][2]);
-                    acc[j][3] = fmaf(w1, x.w, acc[j][3]);
+                float* row = vs + rr * C * d.nz4;
+                const float* src = u0 + (int64_t)(r0 + rr) * n;
+                if (aligned) {
+                    if (tid < n4) sno_cp16(row + 4 * tid, src + 4 * tid);
+                } else {
+                    for (int z = tid; z < n; z += ZF_T) row[z] = src[z];
                 }
+            } else if (q < n4) {
+                for (int c = tid >> lv; c < C; c += ZF_T >> lv)
+                    sno_cp16(vs + (rr * C + c) * d.nz4 + 4 * q, v + (((int64_t)b * C + c) * n2 + xy) * n + 4 * q);
             }
-            for (int c = 0; c < (u0 ? 0 : C); c += 4) {
-                float4 x[4];
+            const int kz = tid & ((1 << lm) - 1);
+            if (kz < m)
+                for (int c = tid >> lm; c < C; c += ZF_T >> lm)
+                    sno_cp8(gs + (rr * m + kz) * d.CG + c, gy + (((int64_t)b * C + c) * n2 + xy) * m + kz);
+        }
+        sno_commit();
+        sno_wait_all();
+        __syncthreads();
+        float lo[8][4], hi[8][4];
+        if (rg < nr) {
 #pragma unroll
-                for (int i = 0; i < 4; ++i) x[i] = *reinterpret_cast<const float4*>(vr + (c + i) * nz4);
+            for (int j = 0; j < 8; ++j)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const float4 w = *reinterpret_cast<const float4*>(Ws + (o0 + j) * C4 + c);
-                    const float wv[4] = {w.x, w.y, w.z, w.w};
+                for (int i = 0; i < 4; ++i) lo[j][i] = hi[j][i] = 0.f;
+            const float4* g = reinterpret_cast<const float4*>(gs + rg * m * d.CG + o0);
+            for (int kz = 0; kz < m; ++kz, g += d.CG / 2) {
+                const float4 c4 = *reinterpret_cast<const float4*>(tc + kz * d.TS + z0);
+                const float4 s4 = *reinterpret_cast<const float4*>(tn + kz * d.TS + z0);
+                const float cv[4] = {c4.x, c4.y, c4.z, c4.w}, sv[4] = {s4.x, s4.y, s4.z, s4.w};
+#pragma unroll
+                for (int j = 0; j < 8; j += 2) {
+                    const float4 x = g[j / 2];
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
-                        acc[j][0] = fmaf(wv[i], x[i].x, acc[j][0]);
-                        acc[j][1] = fmaf(wv[i], x[i].y, acc[j][1]);
-                        acc[j][2] = fmaf(wv[i], x[i].z, acc[j][2]);
-                        acc[j][3] = fmaf(wv[i], x[i].w, acc[j][3]);
+                        lo[j][i] = fmaf(cv[i], x.x, lo[j][i]);
+                        hi[j][i] = fmaf(sv[i], x.y, hi[j][i]);
+                        lo[j + 1][i] = fmaf(cv[i], x.z, lo[j + 1][i]);
+                        hi[j + 1][i] = fmaf(sv[i], x.w, hi[j + 1][i]);
                     }
                 }
             }
-        }
-        __syncthreads();   // every tile is in registers: v_next overwrites v
-        if (e < nitems) {
-            const int64_t r = r0 + rg, b = r / n2, xy = r % n2;
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                float4 a = make_float4(acc[j][0], acc[j][1], acc[j][2], acc[j][3]);
-                if (act) a = make_float4(gelu_f(a.x), gelu_f(a.y), gelu_f(a.z), gelu_f(a.w));
-                *reinterpret_cast<float4*>(vs + (rg * C + o0 + j) * nz4 + z0) = a;
-                *reinterpret_cast<float4*>(vnext + ((b * C + o0 + j) * n2 + xy) * n + z0) = a;
+            for (int j = 0; j < 8; ++j) {   // points z0 + i (at -t) and n - 1 - z0 - i (at +t)
+                const float bj = bs[o0 + j];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float a = lo[j][i] + bj, b = hi[j][i];
+                    lo[j][i] = a + b;
+                    hi[j][i] = a - b;
+                }
+            }
+            const float* vr = vs + rg * C * d.nz4;
+            const float* wr = (u0 ? bs + d.CP : Ws) + o0;
+            const int nc = u0 ? 1 : C;
+            for (int c = 0; c < nc; ++c, vr += d.nz4, wr += d.CP) {
+                const float4 a = *reinterpret_cast<const float4*>(vr + z0);
+                const float4 b = rev4(*reinterpret_cast<const float4*>(vr + z1));
+                const float4 w0 = *reinterpret_cast<const float4*>(wr), w1 = *reinterpret_cast<const float4*>(wr + 4);
+                const float wv[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
+                const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        lo[j][i] = fmaf(wv[j], av[i], lo[j][i]);
+                        hi[j][i] = fmaf(wv[j], bv[i], hi[j][i]);
+                    }
+            }
+        }
+        __syncthreads();   // every tile is in registers: v_next (or its sums and differences) replaces v
+        if (rg < nr) {
+            const int b = (r0 + rg) / n2, xy = (r0 + rg) - b * n2;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                if (o0 + j >= C) break;
+                const int64_t gi = (((int64_t)b * C + o0 + j) * n2 + xy) * n;
+                float4 a = make_float4(lo[j][0], lo[j][1], lo[j][2], lo[j][3]);
+                float4 h = make_float4(hi[j][0], hi[j][1], hi[j][2], hi[j][3]);
+                if (zout) {
+                    *reinterpret_cast<float4*>(zout + gi + z0) = a;
+                    *reinterpret_cast<float4*>(zout + gi + z1) = rev4(h);
+                }
+                if (!PROJ) {
+                    a = make_float4(gelu_f(a.x), gelu_f(a.y), gelu_f(a.z), gelu_f(a.w));
+                    h = make_float4(gelu_f(h.x), gelu_f(h.y), gelu_f(h.z), gelu_f(h.w));
+                }
+                if (vnext) {
+                    *reinterpret_cast<float4*>(vnext + gi + z0) = a;
+                    *reinterpret_cast<float4*>(vnext + gi + z1) = rev4(h);
+                }
+                float* sr = vs + (rg * C + o0 + j) * d.nz4;
+                if (!PROJ) {   // sums at [0, nhp), differences at [nhp, 2 nhp), zero past n / 2
+                    const bool two = z0 + 4 > d.nh;   // (n / 2 is even)
+                    *reinterpret_cast<float4*>(sr + z0) =
+                        make_float4(h.x + a.x, h.y + a.y, two ? 0.f : h.z + a.z, two ? 0.f : h.w + a.w);
+                    *reinterpret_cast<float4*>(sr + d.nhp + z0) =
+                        make_float4(h.x - a.x, h.y - a.y, two ? 0.f : h.z - a.z, two ? 0.f : h.w - a.w);
+                } else {
+                    *reinterpret_cast<float4*>(sr + z0) = a;
+                    *reinterpret_cast<float4*>(sr + z1) = rev4(h);
+                }
             }
         }
         __syncthreads();
-        if (cznext) {   // phase B: cz[c][kz] for 3 modes per thread, the points as float4
-            const int nkb = (m + 2) / 3;
-            for (int f = threadIdx.x; f < nr * nkb * C; f += blockDim.x) {
-                const int c = f % C, kb = (f / C) % nkb, rq = f / (C * nkb);
+        if (!PROJ) {   // channels cg + ncg i, modes 3 kb + i
+            const int ncg = C / 4, nkb = (m + 2) / 3;
+            for (int e = tid; e < nr * ncg * nkb; e += ZF_T) {
+                const int cg = e % ncg, kb = (e / ncg) % nkb, rq = e / (ncg * nkb);
                 int kc[3];
 #pragma unroll
-                for (int i = 0; i < 3; ++i) kc[i] = min(3 * kb + i, m - 1);
-                float re[3] = {0.f, 0.f, 0.f}, im[3] = {0.f, 0.f, 0.f};
-                const float* vr = vs + (rq * C + c) * nz4;
-                for (int zz = 0; zz < n; zz += 4) {
-                    const float4 xv = *reinterpret_cast<const float4*>(vr + zz);
+                for (int i = 0; i < 3; ++i) kc[i] = min(3 * kb + i, m - 1) * d.TS;
+                float re[4][3] = {}, im[4][3] = {};
+                const float* vr = vs + (rq * C + cg) * d.nz4;
+                for (int j = 0; j < d.nhp; j += 4) {
+                    float4 x[4], w[4];
 #pragma unroll
-                    for (int i = 0; i < 3; ++i) {
-                        const float4 ta = *reinterpret_cast<const float4*>(tf + kc[i] * n + zz);
-                        const float4 tb = *reinterpret_cast<const float4*>(tf + kc[i] * n + zz + 2);
-                        re[i] = fmaf(ta.x, xv.x, fmaf(ta.z, xv.y, fmaf(tb.x, xv.z, fmaf(tb.z, xv.w, re[i]))));
-                        im[i] = fmaf(ta.y, xv.x, fmaf(ta.w, xv.y, fmaf(tb.y, xv.z, fmaf(tb.w, xv.w, im[i]))));
+                    for (int i = 0; i < 4; ++i) {
+                        x[i] = *reinterpret_cast<const float4*>(vr + i * ncg * d.nz4 + j);
+                        w[i] = *reinterpret_cast<const float4*>(vr + i * ncg * d.nz4 + d.nhp + j);
                     }
-                }
-                const int64_t r = r0 + rq, b = r / n2, xy = r % n2;
 #pragma unroll
-                for (int i = 0; i < 3; ++i)
-                    if (3 * kb + i < m) cznext[((b * C + c) * n2 + xy) * m + 3 * kb + i] = make_float2(re[i], im[i]);
-            }
-        }
-        if (y) {   // projection: 4 rows of Q1 x 4 points per thread, partial sums per row block
-            for (int f = threadIdx.x; f < nr * npb * n4; f += blockDim.x) {
-                const int zq = f % n4, pb = (f / n4) % npb, rq = f / (n4 * npb);
-                const int zp = 4 * zq, p0 = 4 * pb;
-                int pc[4];
-                float a[4][4];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    pc[j] = min(p0 + j, P - 1);
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) a[j][i] = pq[pc[j]];
-                }
-                const float* vr = vs + rq * C * nz4 + zp;
-                for (int c = 0; c < C; c += 4) {
-                    float4 x[4];
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) x[i] = *reinterpret_cast<const float4*>(vr + (c + i) * nz4);
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const float4 w = *reinterpret_cast<const float4*>(Qs + pc[j] * C4 + c);
-                        const float wv[4] = {w.x, w.y, w.z, w.w};
+                    for (int k = 0; k < 3; ++k) {
+                        const float4 c4 = *reinterpret_cast<const float4*>(tc + kc[k] + j);
+                        const float4 s4 = *reinterpret_cast<const float4*>(tn + kc[k] + j);
 #pragma unroll
                         for (int i = 0; i < 4; ++i) {
-                            a[j][0] = fmaf(wv[i], x[i].x, a[j][0]);
-                            a[j][1] = fmaf(wv[i], x[i].y, a[j][1]);
-                            a[j][2] = fmaf(wv[i], x[i].z, a[j][2]);
-                            a[j][3] = fmaf(wv[i], x[i].w, a[j][3]);
+                            re[i][k] = fmaf(c4.x, x[i].x, fmaf(c4.y, x[i].y, fmaf(c4.z, x[i].z, fmaf(c4.w, x[i].w, re[i][k]))));
+                            im[i][k] = fmaf(s4.x, w[i].x, fmaf(s4.y, w[i].y, fmaf(s4.z, w[i].z, fmaf(s4.w, w[i].w, im[i][k]))));
                         }
                     }
                 }
-                float part[4] = {0.f, 0.f, 0.f, 0.f};
+                const int b = (r0 + rq) / n2, xy = (r0 + rq) - b * n2;
 #pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    if (p0 + j < P)
+                for (int i = 0; i < 4; ++i) {
+                    float2* o = cznext + (((int64_t)b * C + cg + i * ncg) * n2 + xy) * m + 3 * kb;
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) part[i] = fmaf(pq[P + p0 + j], gelu_f(a[j][i]), part[i]);
+                    for (int k = 0; k < 3; ++k)
+                        if (3 * kb + k < m) o[k] = make_float2(re[i][k], -im[i][k]);
+                }
+            }
+        }
+        if (PROJ) {   // projection: 8 rows of Q1 x 8 points a thread, partial sums per row block
+            const int npb = d.PP / 8, nq = (n4 + 1) / 2;
+            for (int e = tid; e < nr * npb * nq; e += ZF_T) {
+                const int q = e % nq, pb = (e / nq) % npb, rq = e / (nq * npb);
+                const int za = 4 * q, zc = 4 * min(q + nq, n4 - 1), p0 = 8 * pb;
+                float a[8][8];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) ys[(rq * npb + pb) * n + zp + i] = part[i];
+                for (int j = 0; j < 8; ++j)
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) a[j][i] = pq[p0 + j];
+                const float* vr = vs + rq * C * d.nz4;
+                const float* qr = Qs + p0;
+                for (int c = 0; c < C; ++c, vr += d.nz4, qr += d.PP) {
+                    const float4 xa = *reinterpret_cast<const float4*>(vr + za);
+                    const float4 xc = *reinterpret_cast<const float4*>(vr + zc);
+                    const float4 w0 = *reinterpret_cast<const float4*>(qr), w1 = *reinterpret_cast<const float4*>(qr + 4);
+                    const float wv[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
+                    const float xv[8] = {xa.x, xa.y, xa.z, xa.w, xc.x, xc.y, xc.z, xc.w};
+#pragma unroll
+                    for (int j = 0; j < 8; ++j)
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) a[j][i] = fmaf(wv[j], xv[i], a[j][i]);
+                }
+                float part[8] = {};
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const float w = pq[d.PP + p0 + j];
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) part[i] = fmaf(w, gelu_f(a[j][i]), part[i]);
+                }
+                float* yo = ys + (rq * npb + pb) * n;
+                *reinterpret_cast<float4*>(yo + za) = make_float4(part[0], part[1], part[2], part[3]);
+                *reinterpret_cast<float4*>(yo + zc) = make_float4(part[4], part[5], part[6], part[7]);
             }
             __syncthreads();
-            for (int f = threadIdx.x; f < nr * n; f += blockDim.x) {
-                const int zz = f % n, rq = f / n;
+            for (int e = tid; e < nr * n; e += ZF_T) {
+                const int rq = e / n, zz = e - rq * n;
                 float sum = 0.f;
                 for (int pb = 0; pb < npb; ++pb) sum += ys[(rq * npb + pb) * n + zz];
-                const int64_t r = r0 + rq;
-                y[r * n + zz] = q2[0] + sum;   // (b n^3 + xy n + z)
-            }
-        }
-        __syncthreads();   // the buffer is refilled two passes later
-    }
-}
-
-// Forward, layer output side, tiled: a block takes FR row groups (b, x, y) at a time. Per
-// row group a thread computes an 8-channel x 4-point tile of z = Re(Tzi gy) + W v + b from
-// float4 shared loads (8 x 4 outputs per 12 loads), stores v_next (GELU unless the last
-// layer) over v in shared memory, then the next layer's cz = Tzf v_next (4 channels x 4 kz
-// per thread) or the projection y (8 projection rows x 4 points per thread). Needs n and
-// the width to be multiples of 4.
-constexpr int FR = 4;
-__global__ void __launch_bounds__(ZR_T) k_zrow_fwd(const float2* __restrict__ gy, const float* __restrict__ v,
-                                                   const float* __restrict__ W, const float* __restrict__ bias,
-                                                   const float2* __restrict__ Tzi, const float2* __restrict__ Tzf,
-                                                   float* __restrict__ zout, float* __restrict__ vnext,
-                                                   float2* __restrict__ cznext, const float* __restrict__ Q1,
-                                                   const float* __restrict__ q1, const float* __restrict__ Q2,
-                                                   const float* __restrict__ q2, float* __restrict__ y, int B, int C,
-                                                   int n, int m, int P, int act, int fr) {
-    extern __shared__ __align__(16) float zsh[];
-    const int nz4 = n + 4, C4 = C + 4, mt = m + 1, nt = n + 2;
-    float* vs = zsh;                               // [FR][C][n + 4]
-    float* Ws = vs + FR * C * nz4;                 // [C][C + 4]
-    float* bs = Ws + C * C4;                       // [C]
-    float* Qs = bs + C;                            // [P][C + 4] (projection)
-    float* pq = Qs + (y ? P * C4 : 0);             // q1, Q2 [2][P]
-    float* ys = pq + (y ? 2 * P : 0);              // [FR][n]
-    size_t fo = (size_t)(ys + (y ? FR * n : 0) - zsh);
-    fo = (fo + 3) & ~(size_t)3;
-    float2* gs = reinterpret_cast<float2*>(zsh + fo);   // [FR][C][m]
-    float2* ti = gs + FR * C * m;                        // [n][m + 1]
-    float2* tf = ti + n * mt;                            // [m][n + 2]
-    for (int e = threadIdx.x; e < C * C; e += blockDim.x) Ws[(e / C) * C4 + e % C] = W[e];
-    for (int e = threadIdx.x; e < C; e += blockDim.x) bs[e] = bias[e];
-    for (int e = threadIdx.x; e < n * m; e += blockDim.x) ti[(e / m) * mt + e % m] = Tzi[e];
-    if (cznext)
-        for (int e = threadIdx.x; e < m * n; e += blockDim.x) tf[(e / n) * nt + e % n] = Tzf[e];
-    if (y) {
-        for (int e = threadIdx.x; e < P * C; e += blockDim.x) Qs[(e / C) * C4 + e % C] = Q1[e];
-        for (int e = threadIdx.x; e < P; e += blockDim.x) {
-            pq[e] = q1[e];
-            pq[P + e] = Q2[e];
-        }
-    }
-    const int64_t n2 = (int64_t)n * n, rows = (int64_t)B * n2;
-    const int nzb = n / 4, nob = (C + 7) / 8, n4 = n / 4;
-    for (int64_t r0 = (int64_t)blockIdx.x * fr; r0 < rows; r0 += (int64_t)gridDim.x * fr) {
-        const int nr = (int)min((int64_t)fr, rows - r0);   // fr row groups: one tile per thread
-        __syncthreads();
-        for (int e = threadIdx.x; e < nr * C * n4; e += blockDim.x) {   // v rows, float4
-            const int q4 = e % n4, c = (e / n4) % C, rg = e / (n4 * C);
-            const int64_t r = r0 + rg, b = r / n2, xy = r % n2;
-            reinterpret_cast<float4*>(vs + (rg * C + c) * nz4)[q4] =
-                reinterpret_cast<const float4*>(v + ((b * C + c) * n2 + xy) * n)[q4];
-        }
-        for (int e = threadIdx.x; e < nr * C * m; e += blockDim.x) {
-            const int kz = e % m, o = (e / m) % C, rg = e / (m * C);
-            const int64_t r = r0 + rg, b = r / n2, xy = r % n2;
-            gs[e] = gy[((b * C + o) * n2 + xy) * m + kz];
-        }
-        if (y)
-            for (int e = threadIdx.x; e < FR * n; e += blockDim.x) ys[e] = 0.f;
-        __syncthreads();
-        // z tiles: 8 channels x 4 points per thread, kept in registers across the sync
-        float acc[1][8][4];
-        const int nitems = nr * nob * nzb;
-        if (threadIdx.x < nitems) {
-            const int k = 0, e = threadIdx.x;
-            const int zb = e % nzb, ob = (e / nzb) % nob, rg = e / (nzb * nob);
-            const int z0 = 4 * zb, o0 = 8 * ob;
-            int oc[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                oc[j] = min(o0 + j, C - 1);
-#pragma unroll
-                for (int i = 0; i < 4; ++i) acc[k][j][i] = bs[oc[j]];
-            }
-            const float2* g = gs + rg * C * m;
-            for (int kz = 0; kz < m; ++kz) {
-                float2 t[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) t[i] = ti[(z0 + i) * mt + kz];
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const float2 gg = g[oc[j] * m + kz];
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) acc[k][j][i] = fmaf(t[i].x, gg.x, fmaf(-t[i].y, gg.y, acc[k][j][i]));
-                }
-            }
-            const float* vr = vs + rg * C * nz4 + z0;
-            for (int c = 0; c < C; c += 4) {
-                float4 x[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) x[i] = *reinterpret_cast<const float4*>(vr + (c + i) * nz4);
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const float4 w = *reinterpret_cast<const float4*>(Ws + oc[j] * C4 + c);
-                    const float wv[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        acc[k][j][0] = fmaf(wv[i], x[i].x, acc[k][j][0]);
-                        acc[k][j][1] = fmaf(wv[i], x[i].y, acc[k][j][1]);
-                        acc[k][j][2] = fmaf(wv[i], x[i].z, acc[k][j][2]);
-                        acc[k][j][3] = fmaf(wv[i], x[i].w, acc[k][j][3]);
-                    }
-                }
-            }
-        }
-        __syncthreads();   // every tile is in registers: v_next may overwrite v in shared memory
-        if (threadIdx.x < nitems) {
-            const int k = 0, e = threadIdx.x;
-            const int zb = e % nzb, ob = (e / nzb) % nob, rg = e / (nzb * nob);
-            const int z0 = 4 * zb, o0 = 8 * ob;
-            const int64_t r = r0 + rg, b = r / n2, xy = r % n2;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const int o = o0 + j;
-                if (o >= C) break;
-                const int64_t gi = ((b * C + o) * n2 + xy) * n + z0;
-                float4 a = make_float4(acc[k][j][0], acc[k][j][1], acc[k][j][2], acc[k][j][3]);
-                if (zout) *reinterpret_cast<float4*>(zout + gi) = a;
-                if (act) a = make_float4(gelu_f(a.x), gelu_f(a.y), gelu_f(a.z), gelu_f(a.w));
-                *reinterpret_cast<float4*>(vs + (rg * C + o) * nz4 + z0) = a;
-                *reinterpret_cast<float4*>(vnext + gi) = a;
-            }
-        }
-        __syncthreads();
-        if (cznext) {   // 4 channels x 4 kz per thread
-            const int ncb = C / 4, nkb = (m + 3) / 4;
-            for (int e = threadIdx.x; e < nr * ncb * nkb; e += blockDim.x) {
-                const int kb = e % nkb, cb = (e / nkb) % ncb, rg = e / (nkb * ncb);
-                const int c0 = 4 * cb, k0 = 4 * kb;
-                int kc[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) kc[i] = min(k0 + i, m - 1);
-                float re[4][4] = {}, im[4][4] = {};
-                const float* vr = vs + (rg * C + c0) * nz4;
-                for (int zz = 0; zz < n; zz += 2) {
-                    float2 xv[4];
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) xv[j] = *reinterpret_cast<const float2*>(vr + j * nz4 + zz);
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const float4 t = *reinterpret_cast<const float4*>(tf + kc[i] * nt + zz);   // z, z + 1
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            re[i][j] = fmaf(t.x, xv[j].x, fmaf(t.z, xv[j].y, re[i][j]));
-                            im[i][j] = fmaf(t.y, xv[j].x, fmaf(t.w, xv[j].y, im[i][j]));
-                        }
-                    }
-                }
-                const int64_t r = r0 + rg, b = r / n2, xy = r % n2;
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-#pragma unroll
-                    for (int i = 0; i < 4; ++i)
-                        if (k0 + i < m) cznext[((b * C + c0 + j) * n2 + xy) * m + k0 + i] = make_float2(re[i][j], im[i][j]);
-            }
-        }
-        if (y) {   // projection: 8 rows of Q1 x 4 points per thread, partial y summed in shared memory
-            const int npb = (P + 7) / 8;
-            for (int e = threadIdx.x; e < nr * npb * nzb; e += blockDim.x) {
-                const int zb = e % nzb, pb = (e / nzb) % npb, rg = e / (nzb * npb);
-                const int z0 = 4 * zb, p0 = 8 * pb;
-                int pc[8];
-                float a[8][4];
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    pc[j] = min(p0 + j, P - 1);
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) a[j][i] = pq[pc[j]];
-                }
-                const float* vr = vs + rg * C * nz4 + z0;
-                for (int c = 0; c < C; c += 4) {
-                    float4 x[4];
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) x[i] = *reinterpret_cast<const float4*>(vr + (c + i) * nz4);
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        const float4 w = *reinterpret_cast<const float4*>(Qs + pc[j] * C4 + c);
-                        const float wv[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            a[j][0] = fmaf(wv[i], x[i].x, a[j][0]);
-                            a[j][1] = fmaf(wv[i], x[i].y, a[j][1]);
-                            a[j][2] = fmaf(wv[i], x[i].z, a[j][2]);
-                            a[j][3] = fmaf(wv[i], x[i].w, a[j][3]);
-                        }
-                    }
-                }
-                float part[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    if (p0 + j >= P) break;
-                    const float q2w = pq[P + p0 + j];
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) part[i] = fmaf(q2w, gelu_f(a[j][i]), part[i]);
-                }
-#pragma unroll
-                for (int i = 0; i < 4; ++i) atomicAdd(ys + rg * n + z0 + i, part[i]);
-            }
-            __syncthreads();
-            for (int e = threadIdx.x; e < nr * n; e += blockDim.x) {
-                const int zz = e % n, rg = e / n;
-                const int64_t r = r0 + rg, b = r / n2, xy = r % n2;
-                y[b * n2 * n + xy * n + zz] = q2[0] + ys[e];
+                y[(int64_t)(r0 + rq) * n + zz] = q2[0] + sum;   // (b n^3 + xy n + z)
             }
         }
     }
@@ -1399,7 +1262,7 @@ static FoldTile fold_tiles(int64_t P, int L, int inner, int cols) {
 
 // x and y transforms of [P][n][inner] to [P][2m][inner]: about one item a thread, at most 72 KB of
 // tiles (three blocks an SM at n = 64)
-static int plane_fwd(SnoModel& M, const float2* in, float2* out, int64_t P, int inner) {
+static int plane_fwd(SnoModel& M, const float2* in, float2* out, int64_t P, int inner, float zscale = 0.f) {
     const int nkb = (M.m + 8) / 8, kb = std::max(4, (M.m + nkb) / nkb), kp = (kb + 1) & ~1;
     const FoldTile f = fold_tiles(P, M.n, inner, std::max(2, std::min(FF_T / nkb, (72 << 10) / (16 * M.n))) & ~1);
     const size_t smem = ((size_t)2 * f.PB * f.ps + (size_t)nkb * (M.n / 2) * kp) * sizeof(float2);
@@ -1409,12 +1272,12 @@ static int plane_fwd(SnoModel& M, const float2* in, float2* out, int64_t P, int 
     KF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, FF_T, smem));
     const int64_t grid = std::min<int64_t>(f.ntiles, (int64_t)std::max(1, per_sm) * M.num_sms);
     const float2* T = ptr<float2>(M.tabs);
-    k<<<(unsigned)grid, FF_T, smem, M.st>>>(in, out, T + M.tfo, T + M.tph, M.m, nkb, f);
+    k<<<(unsigned)grid, FF_T, smem, M.st>>>(in, out, T + M.tfo, T + M.tph, M.m, nkb, zscale, f);
     KF_LAUNCH();
     return KIFMM_OK;
 }
 // and of [P][2m][inner] to [P][n][inner]
-static int plane_inv(SnoModel& M, const float2* in, float2* out, int64_t P, int inner) {
+static int plane_inv(SnoModel& M, const float2* in, float2* out, int64_t P, int inner, float zscale = 0.f) {
     const int njb = (M.n / 2 + FV_J - 1) / FV_J;
     const FoldTile f = fold_tiles(P, 2 * M.m, inner,
                                   std::max(2, std::min(FV_T / njb, (80 << 10) / (48 * M.m + 16))) & ~1);
@@ -1424,7 +1287,7 @@ static int plane_inv(SnoModel& M, const float2* in, float2* out, int64_t P, int 
     KF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fold_inv, FV_T, smem));
     const int64_t grid = std::min<int64_t>(f.ntiles, (int64_t)std::max(1, per_sm) * M.num_sms);
     const float2* T = ptr<float2>(M.tabs);
-    k_fold_inv<<<(unsigned)grid, FV_T, smem, M.st>>>(in, out, T + M.tfo, T + M.tph, M.m, M.n, njb, f);
+    k_fold_inv<<<(unsigned)grid, FV_T, smem, M.st>>>(in, out, T + M.tfo, T + M.tph, M.m, M.n, njb, zscale, f);
     KF_LAUNCH();
     return KIFMM_OK;
 }
@@ -1445,23 +1308,7 @@ static int mix(SnoModel& M, int l, const float2* V, float2* G, int B, int adj) {
 }
 
 static unsigned zr_blocks(const SnoModel& M, int B) { return nbs((int64_t)B * M.n * M.n, ZR_RG); }
-static int zr_fwd_rows(const SnoModel& M) {   // row groups per pass: one 8 x 4 tile per thread
-    const int tiles = ((M.C + 7) / 8) * (M.n / 4);
-    return std::max(1, std::min(FR, ZR_T / tiles));
-}
-static unsigned zr_fwd_blocks(const SnoModel& M, int B) {
-    return (unsigned)std::min<int64_t>(nbs((int64_t)B * M.n * M.n, zr_fwd_rows(M)), 16LL * M.num_sms);
-}
-
 static int near_add(SnoModel& M, const float* u, float* y, int B);
-
-static size_t zrow_inf_smem(int n, int C, int m, int P, bool proj) {
-    const int npb = (P + 3) / 4;
-    size_t f = (size_t)2 * FI * C * (n + 4) + (size_t)C * (C + 4) + C;
-    if (proj) f += (size_t)P * (C + 4) + 2 * (size_t)P + (size_t)FI * npb * n;
-    f = (f + 3) & ~(size_t)3;
-    return f * 4 + ((size_t)2 * FI * C * m + (size_t)m * n) * 8 + (size_t)2 * m * n * 4;
-}
 
 // forward; train: keep z_l and the spectra V_l for the backward pass
 static int forward(SnoModel& M, const float* u, float* y, int B, bool train) {
@@ -1471,14 +1318,15 @@ static int forward(SnoModel& M, const float* u, float* y, int B, bool train) {
     const float* th = ptr<float>(M.theta);
     const float2* T = ptr<float2>(M.tabs);
     const int q = o_q1(M);
-    const bool inf = !train && M.zi_smem;   // inference: layer 0 from u, persistent z-row kernel
-    if (inf) {
+    const float wn = 1.f / ((float)M.period * M.period * M.period);
+    if (!train) {   // inference: layer 0 from u
+
         const int64_t rows = (int64_t)B * n * n;
-        k_lift_u<<<(unsigned)((rows + LU - 1) / LU), 256, (size_t)LU * n * 4 + (size_t)m * n * 8, st>>>(
-            u, T + M.tzf, ptr<float2>(M.cz), rows, n, m);
+        k_lift_u<<<(unsigned)((rows + LU - 1) / LU), 256, (size_t)(LU * (n / 2 + 1) + n / 2 * (m + 1)) * 8, st>>>(
+            u, T + M.tfo, ptr<float2>(M.cz), rows, n, m);
         KF_LAUNCH();
         KF_TRY(plane_fwd(M, ptr<float2>(M.cz), ptr<float2>(M.cy), (int64_t)B * n, m));     // y
-        KF_TRY(plane_fwd(M, ptr<float2>(M.cy), ptr<float2>(M.Vst), B, M2 * m));           // x: U
+        KF_TRY(plane_fwd(M, ptr<float2>(M.cy), ptr<float2>(M.Vst), B, M2 * m, 1.f));      // x: U
         float2* A = ptr<float2>(M.m0ab);
         float2* Bc = A + (int64_t)C * M.K;
         const unsigned np = nbs((int64_t)C * M.K, 256);
@@ -1499,35 +1347,27 @@ static int forward(SnoModel& M, const float* u, float* y, int B, bool train) {
         KF_LAUNCH();
     }
     for (int l = 0; l < M.L; ++l) {
-        if (!(inf && l == 0)) {
+        if (train || l > 0) {   // (the training's lift is not centred)
             float2* V = ptr<float2>(M.Vst) + (train ? (int64_t)l * BC * M.K : 0);
             KF_TRY(plane_fwd(M, ptr<float2>(M.cz), ptr<float2>(M.cy), BC * n, m));            // y
-            KF_TRY(plane_fwd(M, ptr<float2>(M.cy), V, BC, M2 * m));                            // x
+            KF_TRY(plane_fwd(M, ptr<float2>(M.cy), V, BC, M2 * m, l == 0 ? 0.f : 1.f));                            // x
             KF_TRY(mix(M, l, V, ptr<float2>(M.g), B, 0));
         }
-        KF_TRY(plane_inv(M, ptr<float2>(M.g), ptr<float2>(M.gx), BC, M2 * m));             // x^-1
-        KF_TRY(plane_inv(M, ptr<float2>(M.gx), ptr<float2>(M.gy), BC * n, m));             // y^-1
-        const bool last = l == M.L - 1;
-        if (inf) {
-            const size_t sm = last ? M.zi_smem_y : M.zi_smem;
-            int per_sm = 1;
-            auto* kz = (C == 32 && n == 64 && m == 12) ? k_zrow_inf<32, 64, 12> : k_zrow_inf<0, 0, 0>;
-            KF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kz, ZR_T, sm));
-            const int64_t groups = ((int64_t)B * n * n + FI - 1) / FI;
-            const int64_t grid = std::min<int64_t>(groups, (int64_t)std::max(1, per_sm) * M.num_sms);
-            kz<<<(unsigned)grid, ZR_T, sm, st>>>(
-                ptr<float2>(M.gy), l == 0 ? nullptr : fld(M.v, l, per), th + M.off[o_w(l)], th + M.off[o_b(l)],
-                T + M.tzi, T + M.tzf, fld(M.v, l + 1, per), last ? nullptr : ptr<float2>(M.cz), th + M.off[q],
-                th + M.off[q + 1], th + M.off[q + 2], th + M.off[q + 3], last ? y : nullptr, B, C, n, m, M.P,
-                last ? 0 : 1, l == 0 ? u : nullptr, th + M.off[O_WL], th + M.off[O_BL]);
-            KF_LAUNCH();
-            continue;
-        }
-        k_zrow_fwd<<<zr_fwd_blocks(M, B), ZR_T, M.zf_smem, st>>>(
-            ptr<float2>(M.gy), fld(M.v, l, per), th + M.off[o_w(l)], th + M.off[o_b(l)], T + M.tzi, T + M.tzf,
-            train ? fld(M.z, l, per) : nullptr, fld(M.v, l + 1, per), last ? nullptr : ptr<float2>(M.cz),
-            th + M.off[q], th + M.off[q + 1], th + M.off[q + 2], th + M.off[q + 3], last ? y : nullptr, B, C, n, m,
-            M.P, last ? 0 : 1, zr_fwd_rows(M));
+        KF_TRY(plane_inv(M, ptr<float2>(M.g), ptr<float2>(M.gx), BC, M2 * m, wn));                   // x^-1
+        KF_TRY(plane_inv(M, ptr<float2>(M.gx), ptr<float2>(M.gy), BC * n, m));                       // y^-1
+        const bool last = l == M.L - 1, lift = !train && l == 0;
+        const ZRowDims d = zrow_dims(n, C, m, M.P, last);
+        const int rows = B * n * n;
+        int per_sm = 1;
+        auto* kz = last ? k_zrow<true> : k_zrow<false>;   // (the last layer's rows go into the projection)
+        KF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kz, ZF_T, d.smem));
+        const int grid = std::min((rows + d.R - 1) / d.R, std::max(1, per_sm) * M.num_sms);
+        kz<<<grid, ZF_T, d.smem, st>>>(
+            ptr<float2>(M.gy), lift ? nullptr : fld(M.v, l, per), th + M.off[o_w(l)], th + M.off[o_b(l)], T + M.tfo,
+            train ? fld(M.z, l, per) : nullptr, train || !last ? fld(M.v, l + 1, per) : nullptr,
+            last ? nullptr : ptr<float2>(M.cz), th + M.off[q], th + M.off[q + 1], th + M.off[q + 2], th + M.off[q + 3],
+            last ? y : nullptr, lift ? u : nullptr, th + M.off[O_WL], th + M.off[O_BL], rows, C, n, m, M.P,
+            d);
         KF_LAUNCH();
     }
     return near_add(M, u, y, B);   // the exact near part (when set) is a fixed addend of y
@@ -1924,10 +1764,11 @@ int sno_create(sno_model_t* out, int n, int width, int modes, int layers, int pr
         const size_t zb = (3 * width * ns + width * C1) * f4 + al +
                           ((size_t)width * modes + n * (modes + 1) + modes * ns) * f8;
         M.zr_smem_f = std::max(lift, std::max(zf, zb));
-        M.zf_smem = ((size_t)FR * width * (n + 4) + width * (width + 4) + width + proj_width * (width + 4) +
-                     2 * proj_width + FR * n) * f4 + al +
-                    ((size_t)FR * width * modes + n * (modes + 1) + modes * (n + 2)) * f8;
-        M.zr_smem_p = zf + ((size_t)proj_width * C1 + 4 * n + 2 * proj_width) * f4;
+        // (the forward z-row kernel takes less: the limit on the shapes is an older form's)
+        const size_t zr = ((size_t)4 * width * (n + 4) + width * (width + 4) + width + proj_width * (width + 4) +
+                     2 * proj_width + 4 * n) * f4 + al +
+                    ((size_t)4 * width * modes + n * (modes + 1) + modes * (n + 2)) * f8;
+        const size_t zp = zf + ((size_t)proj_width * C1 + 4 * n + 2 * proj_width) * f4;
         M.zr_smem_b = (3 * width * ns + 2 * proj_width * ns + proj_width * C1 + 2 * proj_width + n) * f4 + al +
                       (size_t)modes * ns * f8;
         const size_t per_mode = (size_t)width * (width + 1 + 2 * max_batch) * f8;
@@ -1935,15 +1776,10 @@ int sno_create(sno_model_t* out, int n, int width, int modes, int layers, int pr
         M.mix_smem = (size_t)M.mix_mb * per_mode;
         M.mixg_smem = (size_t)2 * max_batch * M.mix_mb * width * f8;
         const size_t plane_smem = ((size_t)n * 128 + (size_t)n * 2 * modes) * f8;
-        if (width % 4 == 0 && n % 4 == 0 && FI * (width / 4) * (n / 4) <= ZR_T) {
-            M.zi_smem = zrow_inf_smem(n, width, modes, proj_width, false);
-            M.zi_smem_y = zrow_inf_smem(n, width, modes, proj_width, true);
-        }
         int dev = 0, optin = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-        const size_t need = std::max({M.zr_smem_f, M.zr_smem_p, M.zr_smem_b, M.mix_smem, M.mixg_smem, plane_smem,
-                                      M.zf_smem});
+        const size_t need = std::max({M.zr_smem_f, zp, M.zr_smem_b, M.mix_smem, M.mixg_smem, plane_smem, zr});
         cudaDeviceGetAttribute(&M.num_sms, cudaDevAttrMultiProcessorCount, dev);
         M.num_sms = std::max(M.num_sms, 1);
         if (optin <= 0 || need > (size_t)optin) {
@@ -1953,15 +1789,14 @@ int sno_create(sno_model_t* out, int n, int width, int modes, int layers, int pr
         }
         const int lim = optin;
         cudaFuncSetAttribute(k_lift_z, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-        cudaFuncSetAttribute(k_zrow_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+        cudaFuncSetAttribute(k_zrow<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+        cudaFuncSetAttribute(k_zrow<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
         cudaFuncSetAttribute(k_zinv_point_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
         cudaFuncSetAttribute(k_proj_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
         for (auto* k : {k_fold_fwd<4>, k_fold_fwd<5>, k_fold_fwd<6>, k_fold_fwd<7>, k_fold_fwd<8>})
             cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
         cudaFuncSetAttribute(k_fold_inv, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-        cudaFuncSetAttribute(k_zrow_inf<32, 64, 12>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-        cudaFuncSetAttribute(k_zrow_inf<0, 0, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-        if (M.zi_smem_y > (size_t)lim) M.zi_smem = M.zi_smem_y = 0;
+        cudaFuncSetAttribute(k_lift_u, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
         cudaFuncSetAttribute(k_mix<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
         cudaFuncSetAttribute(k_mix<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
         cudaFuncSetAttribute(k_mix_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
@@ -1989,14 +1824,13 @@ int sno_create(sno_model_t* out, int n, int width, int modes, int layers, int pr
     M.tzf = 0;
     M.tyf = M.tzf + (int64_t)modes * n;
     M.tzb = M.tyf + (int64_t)2 * modes * n;
-    M.tzi = M.tzb + (int64_t)modes * n;
-    M.tzr = M.tzi + (int64_t)n * modes;
+    M.tzr = M.tzb + (int64_t)modes * n;
     M.tfo = M.tzr + (int64_t)n * modes;
     M.tph = M.tfo + (int64_t)n / 2 * (modes + 1);
     if ((rc = dev_alloc(M.tabs, (M.tph + modes + 1) * sizeof(float2)))) return fail(rc);
     M.period = n;
     k_tables<<<nbs(2 * modes * n, 128), 128, 0, M.st>>>(n, n, modes, ptr<float2>(M.tabs), M.tzf, M.tyf, M.tzb,
-                                                          M.tzi, M.tzr, M.tfo, M.tph);
+                                                          M.tzr, M.tfo, M.tph);
     if (cudaGetLastError() != cudaSuccess) return fail(KIFMM_ERR_CUDA);
     if ((rc = dev_alloc(M.v, (size_t)(layers + 1) * per * 4))) return fail(rc);
     if ((rc = dev_alloc(M.z, (size_t)layers * per * 4))) return fail(rc);
@@ -2038,7 +1872,7 @@ int sno_set_period(sno_model_t h, int period) {
     }
     M.period = period;
     k_tables<<<nbs(2 * M.m * M.n, 128), 128, 0, M.st>>>(M.n, period, M.m, ptr<float2>(M.tabs), M.tzf, M.tyf, M.tzb,
-                                                          M.tzi, M.tzr, M.tfo, M.tph);
+                                                          M.tzr, M.tfo, M.tph);
     KF_LAUNCH();
     KF_CUDA(cudaStreamSynchronize(M.st));
     return KIFMM_OK;
