@@ -59,7 +59,7 @@ struct SnoModel {
     std::vector<int64_t> off;        // offsets: Wl, bl, then per layer Rr, Ri, W, b, then Q1, q1, Q2, q2
     DevBuf theta, grad, adam_m, adam_v, rbf;   // rbf: BF16 copies of Rr, Ri per layer
     DevBuf tabs;                     // float2 twiddle tables
-    int64_t tzf, tyf, tzb, tzr, tfo, tph;   // table offsets (float2 units)
+    int64_t tzf, tyf, tfo, tph;   // table offsets (float2 units)
     // fields (FP32): v[L+1][B][C][np3], z[L][B][C][np3], dz ping-pong [2][B][C][np3], y and dy [B][np3]
     DevBuf v, z, dz, yb, dy, loss;
     // spectra (float2): cz [B][C][n][n][m], cy / gx [B][C][n][2m][m], gy [B][C][n][n][m],
@@ -68,7 +68,7 @@ struct SnoModel {
     DevBuf m0ab;                     // inference, layer 0: A = R Wl and Bc = (R bl) O, [2][C][K] complex
     DevBuf jt, jref, jorig, jerr;    // photo_solve judge: targets, reference values, caller indices, error
     int mix_mb = 1;                  // modes per block of the mixing kernels
-    size_t zr_smem_f = 0, zr_smem_b = 0, mix_smem = 0, mixg_smem = 0;
+    size_t zr_smem_f = 0, mix_smem = 0, mixg_smem = 0;
     int num_sms = 1;
     int64_t steps = 0;
     int period = 0;                  // N of the transforms (>= n)
@@ -119,22 +119,18 @@ __device__ __forceinline__ float gelu_d(float x) {
     return 0.5f * (1.0f + erff(x * 0.70710678118654752f)) + x * 0.3989422804014327f * expf(-0.5f * x * x);
 }
 
-// Twiddle tables: tzf[kz][z] = e^{-i kz z}, tzb = (w/N^3) e^{-i kz z}, tyf[k][y] = e^{-i k y}
-// (k = 0..2m-1 mapped to {0..m-1} U {N-m..N-1}), tzr[z][kz] = e^{+i kz z},
+// Twiddle tables: tzf[kz][z] = e^{-i kz z}, tyf[k][y] = e^{-i k y} (k = 0..2m-1 mapped to
+// {0..m-1} U {N-m..N-1}),
 // tfo[j][k] = (cos, sin)(k (zc - j)) for j < n / 2 and k = 0..m with zc = (n - 1) / 2,
 // tph[k] = (cos, sin)(k zc) (angles in 2 pi / N units, N the period, grid indices 0..n-1).
-__global__ void k_tables(int n, int N, int m, float2* t, int64_t tzf, int64_t tyf, int64_t tzb, int64_t tzr,
-                         int64_t tfo, int64_t tph) {
+__global__ void k_tables(int n, int N, int m, float2* t, int64_t tzf, int64_t tyf, int64_t tfo, int64_t tph) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const double tw = 6.283185307179586476925286766559 / N;
-    const double n3 = (double)N * N * N;
     auto kxy = [&](int k) { return k < m ? k : N - 2 * m + k; };
     if (i < m * n) {
         int kz = i / n, z = i % n;
         double a = tw * kz * z;
-        double w = (kz == 0 ? 1.0 : 2.0) / n3;
         t[tzf + i] = make_float2((float)cos(a), (float)-sin(a));
-        t[tzb + i] = make_float2((float)(w * cos(a)), (float)(-w * sin(a)));
     }
     if (i < 2 * m * n) {
         int k = i / n, y = i % n;
@@ -149,11 +145,6 @@ __global__ void k_tables(int n, int N, int m, float2* t, int64_t tzf, int64_t ty
     if (i <= m) {
         double a = tw * i * (0.5 * (n - 1));
         t[tph + i] = make_float2((float)cos(a), (float)sin(a));
-    }
-    if (i < n * m) {
-        int z = i / m, kz = i % m;
-        double a = tw * kz * z;
-        t[tzr + i] = make_float2((float)cos(a), (float)sin(a));
     }
 }
 
@@ -606,7 +597,7 @@ __global__ void __launch_bounds__(ZR_T) k_lift_z(const float* __restrict__ u, co
 
 // Forward, layer output side: persistent blocks over R row groups (b, x, y) at a time,
 // z = Re(sum_kz g e^{i kz (z - zc)}) + W v + b with v_next = GELU(z) (or z for the last layer), then the
-// next layer's cz = sum_z e^{-i kz (z - zc)} v_next or the projection y; z itself is stored when zout is
+// next layer's cz = sum_z e^{-i kz (z - zc)} v_next or the projection y; z itself is stored when zio is
 // given (training). Layer 0 of the inference takes W v0 + b = (W Wl) u + (W bl + b) from u.
 // The transforms are folded about the row's centre zc = (n - 1) / 2 as in k_fold_fwd (half the FMAs; the
 // phases e^{+-i kz zc} and the weights are in the spectra). A thread computes 8 channels x 4 point pairs:
@@ -616,7 +607,10 @@ __global__ void __launch_bounds__(ZR_T) k_lift_z(const float* __restrict__ u, co
 // blocks an SM cover each other's loads: bound by FP32 issue (FMAs and GELU's erf).
 // One GB300, 32 fields of 64^3 at width 32 and 12 modes: layers 1 and 2 2.28 -> 1.25 ms each,
 // the last with the projection 2.27 -> 1.92 ms, layer 0 0.87 ms; the four launches 6.83 -> 5.3 ms.
+// The backward pass runs the same rows with W transposed: dv = Re(sum_kz g e^{i kz (z - zc)}) + W^T dz, then
+// dz_prev = dv GELU'(z_prev) and its transform (layer 0: dv alone, zio and cznext null).
 constexpr int ZF_T = 128;
+enum { ZR_FWD = 0, ZR_PROJ = 1, ZR_BWD = 2 };   // k_zrow's MODE; zio: z written (forward), z_prev read (backward)
 struct ZRowDims {
     int nh, nhp, nzb, nob, CP, CG, nz4, TS, PP, R;   // (see zrow_dims)
     size_t smem;
@@ -641,16 +635,17 @@ static ZRowDims zrow_dims(int n, int C, int m, int P, bool proj) {
     return d;
 }
 __device__ __forceinline__ float4 rev4(float4 a) { return make_float4(a.w, a.z, a.y, a.x); }
-template <bool PROJ>
+template <int MODE>
 __global__ void __launch_bounds__(ZF_T, 3) k_zrow(const float2* __restrict__ gy, const float* __restrict__ v,
                                                   const float* __restrict__ W, const float* __restrict__ bias,
-                                                  const float2* __restrict__ tfo, float* __restrict__ zout,
+                                                  const float2* __restrict__ tfo, float* __restrict__ zio,
                                                   float* __restrict__ vnext, float2* __restrict__ cznext,
                                                   const float* __restrict__ Q1, const float* __restrict__ q1,
                                                   const float* __restrict__ Q2, const float* __restrict__ q2,
                                                   float* __restrict__ y, const float* __restrict__ u0,
                                                   const float* __restrict__ Wl, const float* __restrict__ bl, int rows,
                                                   int C, int n, int m, int P, ZRowDims d) {
+    constexpr bool PROJ = MODE == ZR_PROJ, BWD = MODE == ZR_BWD;
     extern __shared__ __align__(16) float zsh[];
     float* vs = zsh;                                              // [R][C][n + 4]
     float* Ws = vs + d.R * C * d.nz4;                             // [C][CP], transposed
@@ -664,10 +659,10 @@ __global__ void __launch_bounds__(ZF_T, 3) k_zrow(const float2* __restrict__ gy,
     const int tid = threadIdx.x, n4 = n / 4, n2 = n * n;
     for (int e = tid; e < C * d.CP; e += ZF_T) {
         const int c = e / d.CP, o = e - c * d.CP;
-        Ws[e] = o < C ? W[o * C + c] : 0.f;
+        Ws[e] = o < C ? W[BWD ? c * C + o : o * C + c] : 0.f;
     }
     for (int o = tid; o < d.CP; o += ZF_T) {
-        float w0 = o < C ? bias[o] : 0.f, w1 = 0.f;
+        float w0 = !BWD && o < C ? bias[o] : 0.f, w1 = 0.f;
         if (u0 && o < C)
             for (int c = 0; c < C; ++c) {
                 w1 = fmaf(W[o * C + c], Wl[c], w1);
@@ -783,11 +778,18 @@ __global__ void __launch_bounds__(ZF_T, 3) k_zrow(const float2* __restrict__ gy,
                 const int64_t gi = (((int64_t)b * C + o0 + j) * n2 + xy) * n;
                 float4 a = make_float4(lo[j][0], lo[j][1], lo[j][2], lo[j][3]);
                 float4 h = make_float4(hi[j][0], hi[j][1], hi[j][2], hi[j][3]);
-                if (zout) {
-                    *reinterpret_cast<float4*>(zout + gi + z0) = a;
-                    *reinterpret_cast<float4*>(zout + gi + z1) = rev4(h);
+                if (BWD) {
+                    if (zio) {
+                        const float4 x = *reinterpret_cast<const float4*>(zio + gi + z0);
+                        const float4 w = rev4(*reinterpret_cast<const float4*>(zio + gi + z1));
+                        a = make_float4(a.x * gelu_d(x.x), a.y * gelu_d(x.y), a.z * gelu_d(x.z), a.w * gelu_d(x.w));
+                        h = make_float4(h.x * gelu_d(w.x), h.y * gelu_d(w.y), h.z * gelu_d(w.z), h.w * gelu_d(w.w));
+                    }
+                } else if (zio) {
+                    *reinterpret_cast<float4*>(zio + gi + z0) = a;
+                    *reinterpret_cast<float4*>(zio + gi + z1) = rev4(h);
                 }
-                if (!PROJ) {
+                if (MODE == ZR_FWD) {
                     a = make_float4(gelu_f(a.x), gelu_f(a.y), gelu_f(a.z), gelu_f(a.w));
                     h = make_float4(gelu_f(h.x), gelu_f(h.y), gelu_f(h.z), gelu_f(h.w));
                 }
@@ -809,7 +811,7 @@ __global__ void __launch_bounds__(ZF_T, 3) k_zrow(const float2* __restrict__ gy,
             }
         }
         __syncthreads();
-        if (!PROJ) {   // channels cg + ncg i, modes 3 kb + i
+        if (!PROJ && cznext) {   // channels cg + ncg i, modes 3 kb + i
             const int ncg = C / 4, nkb = (m + 2) / 3;
             for (int e = tid; e < nr * ncg * nkb; e += ZF_T) {
                 const int cg = e % ncg, kb = (e / ncg) % nkb, rq = e / (ncg * nkb);
@@ -891,313 +893,259 @@ __global__ void __launch_bounds__(ZF_T, 3) k_zrow(const float2* __restrict__ gy,
     }
 }
 
-// Sum over the row of X[i][z] Y[j][z] for a thread's 2 x 2 tiles of (i, j) (i < NI, j < NJ),
-// accumulated into acc[4 * t + 2 * di + dj] for tile t = threadIdx.x + t * ZR_T.
-template <int NT>
-__device__ __forceinline__ void tile_sums(const float* X, const float* Y, int NI, int NJ, int n, float* acc) {
-    const int ns = n + 1, nti = (NI + 1) / 2, ntj = (NJ + 1) / 2;
+// ---- backward: the weights' gradients are sums over all points, C x C or P x C at a time. Persistent
+// blocks walk chunks of GP points with 4 x 4 tiles of the sum in registers; where the tiles are fewer
+// than the threads, the chunk's points are split over 2^k lanes a tile (added by shuffles at the end),
+// and a block adds its sums to the gradient once (the row-by-row form added 16384 times 4 rows' sums).
+constexpr int GP = 64;            // points a chunk (n^3 is a multiple of 64)
+constexpr int GPS = GP + 4;       // a channel's row in shared memory
+constexpr int GD_T = 256;
+__device__ __host__ inline int grad_splits(int tiles) {   // lanes a tile, a power of two up to GP / 4
+    int S = GP / 4;
+    while (S > 1 && tiles * S > GD_T) S /= 2;
+    return S;
+}
+// acc[4 i + j] += sum over the lane's points of X[i][.] Y[j][.]
+__device__ __forceinline__ void grad_tile(const float* X, const float* Y, int s, int S, float* acc) {
+    for (int q = 4 * s; q < GP; q += 4 * S) {
+        float4 x[4], w[4];
 #pragma unroll
-    for (int t = 0; t < NT; ++t) {
-        const int tt = threadIdx.x + t * ZR_T;
-        if (tt >= nti * ntj) break;
-        const int i0 = 2 * (tt / ntj), j0 = 2 * (tt % ntj);
-        const float* x0 = X + i0 * ns;
-        const float* x1 = X + min(i0 + 1, NI - 1) * ns;
-        const float* y0 = Y + j0 * ns;
-        const float* y1 = Y + min(j0 + 1, NJ - 1) * ns;
-        float s00 = 0.f, s01 = 0.f, s10 = 0.f, s11 = 0.f;
-        for (int zz = 0; zz < n; ++zz) {
-            const float a = x0[zz], bb = x1[zz], c = y0[zz], d = y1[zz];
-            s00 = fmaf(a, c, s00);
-            s01 = fmaf(a, d, s01);
-            s10 = fmaf(bb, c, s10);
-            s11 = fmaf(bb, d, s11);
+        for (int i = 0; i < 4; ++i) {
+            x[i] = *reinterpret_cast<const float4*>(X + i * GPS + q);
+            w[i] = *reinterpret_cast<const float4*>(Y + i * GPS + q);
         }
-        acc[4 * t] += s00;
-        acc[4 * t + 1] += s01;
-        acc[4 * t + 2] += s10;
-        acc[4 * t + 3] += s11;
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                acc[4 * i + j] = fmaf(x[i].x, w[j].x, fmaf(x[i].y, w[j].y, fmaf(x[i].z, w[j].z, fmaf(x[i].w, w[j].w, acc[4 * i + j]))));
     }
 }
-template <int NT>
-__device__ __forceinline__ void tile_flush(const float* acc, int NI, int NJ, float* g) {
-    const int nti = (NI + 1) / 2, ntj = (NJ + 1) / 2;
-#pragma unroll
-    for (int t = 0; t < NT; ++t) {
-        const int tt = threadIdx.x + t * ZR_T;
-        if (tt >= nti * ntj) break;
-        const int i0 = 2 * (tt / ntj), j0 = 2 * (tt % ntj);
-#pragma unroll
-        for (int di = 0; di < 2; ++di)
-#pragma unroll
-            for (int dj = 0; dj < 2; ++dj)
-                if (i0 + di < NI && j0 + dj < NJ) atomicAdd(g + (i0 + di) * NJ + j0 + dj, acc[4 * t + 2 * di + dj]);
-    }
-}
-constexpr int NT_Q = (MAXP / 2) * (MAXC / 2) / ZR_T;   // 2 x 2 tiles per thread of a P x C sum
-constexpr int NT_W = (MAXC / 2) * (MAXC / 2) / ZR_T;   // and of a C x C sum
-
-// backward of the projection and of the last layer's pointwise part (no GELU there):
-// a = Q1 v_L + q1, h = GELU(a), da = dy Q2 GELU'(a), dz_{L-1} = Q1^T da; czb = Tzb dz_{L-1};
-// block partial sums of dQ1, dq1, dQ2, dq2, dW_{L-1}, db_{L-1} added atomically.
-__global__ void __launch_bounds__(ZR_T) k_proj_bwd(const float* __restrict__ vL, const float* __restrict__ vLm1,
-                                                   const float* __restrict__ dy, const float* __restrict__ Q1,
-                                                   const float* __restrict__ q1, const float* __restrict__ Q2,
-                                                   const float2* __restrict__ Tzb, float* __restrict__ dz,
-                                                   float2* __restrict__ czb, float* gQ1, float* gq1, float* gQ2,
-                                                   float* gq2, float* gW, float* gb, int B, int C, int n, int m, int P) {
-    extern __shared__ float zsh[];
-    const int ns = n + 1, C1 = C + 1;
-    float* vs = zsh;                 // v_L [C][n + 1]
-    float* ws = vs + C * ns;         // v_{L-1} [C][n + 1]
-    float* ds = ws + C * ns;         // dz [C][n + 1]
-    float* das = ds + C * ns;        // da [P][n + 1]
-    float* hs = das + P * ns;        // h [P][n + 1]
-    float* Qs = hs + P * ns;         // Q1 [P][C + 1]
-    float* pq = Qs + P * C1;         // q1, Q2 [2][P]
-    float* dys = pq + 2 * P;         // dy [n]
-    size_t fo = (size_t)(dys + n - zsh);
-    fo = (fo + 1) & ~(size_t)1;
-    float2* tb = reinterpret_cast<float2*>(zsh + fo);   // [m][n + 1]
-    for (int e = threadIdx.x; e < P * C; e += blockDim.x) Qs[(e / C) * C1 + e % C] = Q1[e];
-    for (int e = threadIdx.x; e < P; e += blockDim.x) {
-        pq[e] = q1[e];
-        pq[P + e] = Q2[e];
-    }
-    for (int e = threadIdx.x; e < m * n; e += blockDim.x) tb[(e / n) * ns + e % n] = Tzb[e];
-    float aQ1[4 * NT_Q], aW[4 * NT_W];
-#pragma unroll
-    for (int j = 0; j < 4 * NT_Q; ++j) aQ1[j] = 0.f;
-#pragma unroll
-    for (int j = 0; j < 4 * NT_W; ++j) aW[j] = 0.f;
-    float aq1 = 0.f, aQ2 = 0.f, ab = 0.f, aq2 = 0.f;   // thread < P: q1[t], Q2[t]; thread < C: b[t]; thread 0: q2
-    const int64_t n2 = (int64_t)n * n, rows = (int64_t)B * n2;
-    const int zb = (n + 1) / 2;
-    for (int64_t r = (int64_t)blockIdx.x * ZR_RG; r < min(rows, (int64_t)(blockIdx.x + 1) * ZR_RG); ++r) {
-        const int64_t b = r / n2, xy = r % n2;
-        __syncthreads();
-        for (int e = threadIdx.x; e < C * n; e += blockDim.x) {
-            const int c = e / n, zz = e % n;
-            const int64_t gi = ((b * C + c) * n2 + xy) * n + zz;
-            vs[c * ns + zz] = vL[gi];
-            ws[c * ns + zz] = vLm1[gi];
-        }
-        for (int e = threadIdx.x; e < n; e += blockDim.x) dys[e] = dy[b * n2 * n + xy * n + e];
-        __syncthreads();
-        // a for projection rows p0..p0+3 at points z0, z1
-        for (int e = threadIdx.x; e < ((P + 3) / 4) * zb; e += blockDim.x) {
-            const int z0 = e % zb, p0 = 4 * (e / zb);
-            const int z1 = z0 + zb < n ? z0 + zb : z0;
-            int pc[4];
-            float a0[4], a1[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                pc[u] = min(p0 + u, P - 1);
-                a0[u] = a1[u] = pq[pc[u]];
-            }
-            for (int c = 0; c < C; ++c) {
-                const float x0 = vs[c * ns + z0], x1 = vs[c * ns + z1];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const float w = Qs[pc[u] * C1 + c];
-                    a0[u] = fmaf(w, x0, a0[u]);
-                    a1[u] = fmaf(w, x1, a1[u]);
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                if (p0 + u >= P) break;
-                const int p = p0 + u;
-                hs[p * ns + z0] = gelu_f(a0[u]);
-                das[p * ns + z0] = dys[z0] * pq[P + p] * gelu_d(a0[u]);
-                if (z1 != z0) {
-                    hs[p * ns + z1] = gelu_f(a1[u]);
-                    das[p * ns + z1] = dys[z1] * pq[P + p] * gelu_d(a1[u]);
-                }
-            }
-        }
-        __syncthreads();
-        // dz = Q1^T da for channels c0..c0+3 at points z0, z1
-        for (int e = threadIdx.x; e < ((C + 3) / 4) * zb; e += blockDim.x) {
-            const int z0 = e % zb, c0 = 4 * (e / zb);
-            const int z1 = z0 + zb < n ? z0 + zb : z0;
-            int cc[4];
-            float a0[4] = {0.f, 0.f, 0.f, 0.f}, a1[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-            for (int u = 0; u < 4; ++u) cc[u] = min(c0 + u, C - 1);
-            for (int p = 0; p < P; ++p) {
-                const float x0 = das[p * ns + z0], x1 = das[p * ns + z1];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const float w = Qs[p * C1 + cc[u]];
-                    a0[u] = fmaf(w, x0, a0[u]);
-                    a1[u] = fmaf(w, x1, a1[u]);
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                if (c0 + u >= C) break;
-                const int c = c0 + u;
-                const int64_t g0 = ((b * C + c) * n2 + xy) * n;
-                ds[c * ns + z0] = a0[u];
-                dz[g0 + z0] = a0[u];
-                if (z1 != z0) {
-                    ds[c * ns + z1] = a1[u];
-                    dz[g0 + z1] = a1[u];
-                }
-            }
-        }
-        __syncthreads();
-        zfwd_rows(ds, tb, C, n, m, czb + (b * C * n2 + xy) * m, n2 * m);
-        tile_sums<NT_Q>(das, vs, P, C, n, aQ1);    // dQ1[p][c] += sum_z da[p][z] v_L[c][z]
-        tile_sums<NT_W>(ds, ws, C, C, n, aW);      // dW[o][c] += sum_z dz[o][z] v_{L-1}[c][z]
-        if (threadIdx.x < P) {
-            float s1 = 0.f, s2 = 0.f;
-            for (int zz = 0; zz < n; ++zz) {
-                s1 += das[threadIdx.x * ns + zz];
-                s2 = fmaf(dys[zz], hs[threadIdx.x * ns + zz], s2);
-            }
-            aq1 += s1;
-            aQ2 += s2;
-        }
-        if (threadIdx.x < C) {
-            float s = 0.f;
-            for (int zz = 0; zz < n; ++zz) s += ds[threadIdx.x * ns + zz];
-            ab += s;
-        }
-        if (threadIdx.x == 0) {
-            float s = 0.f;
-            for (int zz = 0; zz < n; ++zz) s += dys[zz];
-            aq2 += s;
-        }
-    }
-    tile_flush<NT_Q>(aQ1, P, C, gQ1);
-    tile_flush<NT_W>(aW, C, C, gW);
-    if (threadIdx.x < P) {
-        atomicAdd(gq1 + threadIdx.x, aq1);
-        atomicAdd(gQ2 + threadIdx.x, aQ2);
-    }
-    if (threadIdx.x < C) atomicAdd(gb + threadIdx.x, ab);
-    if (threadIdx.x == 0) atomicAdd(gq2, aq2);
+__device__ __forceinline__ float lane_sum(float a, int S) {   // over S consecutive lanes (a power of two)
+    for (int o = 1; o < S; o *= 2) a += __shfl_xor_sync(0xffffffffu, a, o);
+    return a;
 }
 
-// backward through layer l's output side: dv_l = Re(Tzr gyb) + W_l^T dz_l. For l > 0:
-// dz_{l-1} = dv_l GELU'(z_{l-1}), czb = Tzb dz_{l-1}, partial sums of dW_{l-1}, db_{l-1};
-// for l == 0: partial sums of the lift gradients (dWl from u, dbl).
-__global__ void __launch_bounds__(ZR_T) k_zinv_point_bwd(const float2* __restrict__ gyb, const float* __restrict__ dzl,
-                                                         const float* __restrict__ W, const float2* __restrict__ Tzr,
-                                                         const float* __restrict__ zprev, const float* __restrict__ vprev,
-                                                         const float2* __restrict__ Tzb, float* __restrict__ dzprev,
-                                                         float2* __restrict__ czb, float* gW, float* gb,
-                                                         const float* __restrict__ u, float* gWl, float* gbl, int B,
-                                                         int C, int n, int m) {
-    extern __shared__ float zsh[];
-    const int ns = n + 1, C1 = C + 1;
-    const bool first = (zprev == nullptr);   // l == 0
-    float* ds = zsh;                 // dz_l [C][n + 1]
-    float* dn = ds + C * ns;         // dv_l, then dz_{l-1} [C][n + 1]
-    float* ws = dn + C * ns;         // v_{l-1} or u [C][n + 1]
-    float* Ws = ws + C * ns;         // W_l [C][C + 1]
-    size_t fo = (size_t)(Ws + C * C1 - zsh);
-    fo = (fo + 1) & ~(size_t)1;
-    float2* gs = reinterpret_cast<float2*>(zsh + fo);   // [C][m]
-    float2* tr = gs + C * m;                            // [n][m + 1]
-    float2* tb = tr + n * (m + 1);                      // [m][n + 1]
-    for (int e = threadIdx.x; e < C * C; e += blockDim.x) Ws[(e / C) * C1 + e % C] = W[e];
-    for (int e = threadIdx.x; e < n * m; e += blockDim.x) tr[(e / m) * (m + 1) + e % m] = Tzr[e];
-    if (!first)
-        for (int e = threadIdx.x; e < m * n; e += blockDim.x) tb[(e / n) * ns + e % n] = Tzb[e];
-    float aW[4 * NT_W];
-#pragma unroll
-    for (int j = 0; j < 4 * NT_W; ++j) aW[j] = 0.f;
-    float ab = 0.f, aw1 = 0.f;
-    const int64_t n2 = (int64_t)n * n, rows = (int64_t)B * n2;
-    const int zb = (n + 1) / 2;
-    for (int64_t r = (int64_t)blockIdx.x * ZR_RG; r < min(rows, (int64_t)(blockIdx.x + 1) * ZR_RG); ++r) {
-        const int64_t b = r / n2, xy = r % n2;
-        __syncthreads();
-        for (int e = threadIdx.x; e < C * n; e += blockDim.x) {
-            const int c = e / n, zz = e % n;
-            const int64_t gi = ((b * C + c) * n2 + xy) * n + zz;
-            ds[c * ns + zz] = dzl[gi];
-            if (!first) ws[c * ns + zz] = vprev[gi];
+// dW[o][c] += sum_pt dz[o][pt] v[c][pt], db[o] += sum_pt dz[o][pt]: reads both fields once, the next
+// chunk on its way. Width 16, 4 fields of 64^3: 134 MB, 60 us at worst (4 layers 235 us).
+__global__ void __launch_bounds__(GD_T) k_grad_w(const float* __restrict__ dz, const float* __restrict__ v, float* gW,
+                                                 float* gb, int B, int C, int64_t np3) {
+    extern __shared__ __align__(16) float zsh[];   // two buffers of dz [C][GPS], v [C][GPS]
+    const int nt = C / 4, tiles = nt * nt, S = grad_splits(tiles);
+    const int s = threadIdx.x % S, t = threadIdx.x / S;
+    const int i0 = 4 * (t / nt), j0 = 4 * (t % nt);
+    const int64_t per = np3 / GP, nchunk = per * B;
+    auto issue = [&](int64_t k, float* dst) {
+        const int64_t b = k / per, p = (k - b * per) * GP;
+        const int q = threadIdx.x % (GP / 4);
+        for (int c = threadIdx.x / (GP / 4); c < C; c += GD_T / (GP / 4)) {
+            const int64_t g = (b * C + c) * np3 + p + 4 * q;
+            sno_cp16(dst + c * GPS + 4 * q, dz + g);
+            sno_cp16(dst + (C + c) * GPS + 4 * q, v + g);
         }
-        if (first)
-            for (int e = threadIdx.x; e < n; e += blockDim.x) ws[e] = u[b * n2 * n + xy * n + e];
-        for (int e = threadIdx.x; e < C * m; e += blockDim.x) {
-            const int c = e / m, kz = e % m;
-            gs[e] = gyb[((b * C + c) * n2 + xy) * m + kz];
-        }
-        __syncthreads();
-        // dv for channels c0..c0+3 at points z0, z1
-        for (int e = threadIdx.x; e < ((C + 3) / 4) * zb; e += blockDim.x) {
-            const int z0 = e % zb, c0 = 4 * (e / zb);
-            const int z1 = z0 + zb < n ? z0 + zb : z0;
-            int cc[4];
-            float a0[4] = {0.f, 0.f, 0.f, 0.f}, a1[4] = {0.f, 0.f, 0.f, 0.f};
+    };
+    float acc[16], ab[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-            for (int uu = 0; uu < 4; ++uu) cc[uu] = min(c0 + uu, C - 1);
-            const float2* t0 = tr + z0 * (m + 1);
-            const float2* t1 = tr + z1 * (m + 1);
-            for (int kz = 0; kz < m; ++kz) {
-                const float2 ta = t0[kz], tb2 = t1[kz];
+    for (int i = 0; i < 16; ++i) acc[i] = 0.f;
+    int64_t k = blockIdx.x;
+    if (k < nchunk) issue(k, zsh);
+    sno_commit();
+    for (int it = 0; k < nchunk; k += gridDim.x, ++it) {
+        sno_wait_all();
+        __syncthreads();   // the chunk is there, and the other buffer has been read
+        if (k + gridDim.x < nchunk) issue(k + gridDim.x, zsh + ((it + 1) & 1) * 2 * C * GPS);
+        sno_commit();
+        const float* X = zsh + (it & 1) * 2 * C * GPS;
+        if (t < tiles) {
+            grad_tile(X + i0 * GPS, X + (C + j0) * GPS, s, S, acc);
+            if (j0 == 0)
+                for (int q = 4 * s; q < GP; q += 4 * S)
 #pragma unroll
-                for (int uu = 0; uu < 4; ++uu) {
-                    const float2 g = gs[cc[uu] * m + kz];
-                    a0[uu] = fmaf(ta.x, g.x, fmaf(-ta.y, g.y, a0[uu]));
-                    a1[uu] = fmaf(tb2.x, g.x, fmaf(-tb2.y, g.y, a1[uu]));
-                }
-            }
-            for (int o = 0; o < C; ++o) {
-                const float x0 = ds[o * ns + z0], x1 = ds[o * ns + z1];
-#pragma unroll
-                for (int uu = 0; uu < 4; ++uu) {
-                    const float w = Ws[o * C1 + cc[uu]];
-                    a0[uu] = fmaf(w, x0, a0[uu]);
-                    a1[uu] = fmaf(w, x1, a1[uu]);
-                }
-            }
-#pragma unroll
-            for (int uu = 0; uu < 4; ++uu) {
-                if (c0 + uu >= C) break;
-                const int c = c0 + uu;
-                const int64_t g0 = ((b * C + c) * n2 + xy) * n;
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    if (h == 1 && z1 == z0) break;
-                    const int zz = h ? z1 : z0;
-                    float av = h ? a1[uu] : a0[uu];
-                    if (!first) {
-                        av *= gelu_d(zprev[g0 + zz]);
-                        dzprev[g0 + zz] = av;
+                    for (int i = 0; i < 4; ++i) {
+                        const float4 x = *reinterpret_cast<const float4*>(X + (i0 + i) * GPS + q);
+                        ab[i] += (x.x + x.y) + (x.z + x.w);
                     }
-                    dn[c * ns + zz] = av;
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 16; ++i) acc[i] = lane_sum(acc[i], S);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) ab[i] = lane_sum(ab[i], S);
+    if (t >= tiles || s) return;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) atomicAdd(gW + (i0 + i / 4) * C + j0 + i % 4, acc[i]);
+    if (j0 == 0)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) atomicAdd(gb + i0 + i, ab[i]);
+}
+
+// the lift's gradients: dWl[c] += sum_pt dv[c][pt] u[pt], dbl[c] += sum_pt dv[c][pt]; blockIdx.y = c
+__global__ void __launch_bounds__(256) k_grad_lift(const float* __restrict__ dv, const float* __restrict__ u,
+                                                   float* gWl, float* gbl, int B, int C, int64_t np3) {
+    __shared__ float red[2][8];
+    const int c = blockIdx.y;
+    float sw = 0.f, sb = 0.f;
+    for (int b = 0; b < B; ++b) {
+        const float4* d = reinterpret_cast<const float4*>(dv + ((int64_t)b * C + c) * np3);
+        const float* x = u + b * np3;
+        for (int64_t e = (int64_t)blockIdx.x * 256 + threadIdx.x; e < np3 / 4; e += (int64_t)gridDim.x * 256) {
+            const float4 a = d[e];
+            sw = fmaf(a.x, x[4 * e], fmaf(a.y, x[4 * e + 1], fmaf(a.z, x[4 * e + 2], fmaf(a.w, x[4 * e + 3], sw))));
+            sb += (a.x + a.y) + (a.z + a.w);
+        }
+    }
+    sw = lane_sum(sw, 32);
+    sb = lane_sum(sb, 32);
+    if (threadIdx.x % 32 == 0) {
+        red[0][threadIdx.x / 32] = sw;
+        red[1][threadIdx.x / 32] = sb;
+    }
+    __syncthreads();
+    if (threadIdx.x < 2) {
+        float a = 0.f;
+        for (int w = 0; w < 8; ++w) a += red[threadIdx.x][w];
+        atomicAdd((threadIdx.x ? gbl : gWl) + c, a);
+    }
+}
+
+// backward of the projection: a = Q1 v_L + q1, h = GELU(a), da = dy Q2 GELU'(a), dz_{L-1} = Q1^T da, and the
+// sums dQ1 = da v_L, dq1 = da, dQ2 = dy h, dq2 = dy over all points. Per chunk of GP points: a in tiles of
+// 8 rows of Q1 x 4 points a thread, da through shared memory, dz in tiles of 4 channels x 4 points, dQ1 as in
+// k_grad_w. Bound by FP32 issue. Width 16, 64 rows, 4 fields of 64^3: 835 -> 408 us (the row-by-row
+// form with the last layer's dW and transform in it; those take 60 us each apart).
+constexpr int GQ_TILES = (MAXP / 4) * (MAXC / 4) / GD_T;   // 4 x 4 tiles of dQ1 a thread, at most
+struct ProjDims {
+    int PP, C4;   // rows of Q1 in blocks of 8, row stride of Q1 [p][c]
+    size_t smem;
+};
+static ProjDims proj_dims(int C, int P) {
+    ProjDims d;
+    d.PP = (P + 7) & ~7;
+    d.C4 = C + 4;
+    d.smem = ((size_t)C * GPS + (size_t)d.PP * GPS + (size_t)C * d.PP + (size_t)d.PP * d.C4 + 2 * d.PP + GP) * 4;
+    return d;
+}
+__global__ void __launch_bounds__(GD_T) k_proj_bwd(const float* __restrict__ vL, const float* __restrict__ dy,
+                                                   const float* __restrict__ Q1, const float* __restrict__ q1,
+                                                   const float* __restrict__ Q2, float* __restrict__ dz, float* gQ1,
+                                                   float* gq1, float* gQ2, float* gq2, int B, int C, int P, int64_t np3,
+                                                   ProjDims d) {
+    extern __shared__ __align__(16) float zsh[];
+    float* vs = zsh;                    // v_L [C][GPS]
+    float* das = vs + C * GPS;          // da [PP][GPS]
+    float* Qt = das + d.PP * GPS;       // Q1 transposed [C][PP]
+    float* Qs = Qt + C * d.PP;          // Q1 [PP][C4]
+    float* pq = Qs + d.PP * d.C4;       // q1, Q2 [2][PP]
+    float* dys = pq + 2 * d.PP;         // dy [GP]
+    const int tid = threadIdx.x;
+    for (int e = tid; e < d.PP * C; e += GD_T) {
+        const int p = e / C, c = e - p * C;
+        const float w = p < P ? Q1[e] : 0.f;
+        Qt[c * d.PP + p] = w;
+        Qs[p * d.C4 + c] = w;
+    }
+    for (int p = tid; p < d.PP; p += GD_T) {
+        pq[p] = p < P ? q1[p] : 0.f;
+        pq[d.PP + p] = p < P ? Q2[p] : 0.f;
+    }
+    constexpr int NZ = GP / 4;                  // blocks of 4 points
+    const int nt = C / 4, tiles = d.PP / 4 * nt, S = grad_splits(tiles), s = tid % S;
+    const int zb = tid % NZ, pb = tid / NZ;     // (PP / 8 <= 16 = GD_T / NZ blocks of 8 rows)
+    const int z0 = 4 * zb, p0 = 8 * pb;
+    float aQ1[GQ_TILES][16], aq1[8], aQ2[8], aq2 = 0.f;
+#pragma unroll
+    for (int k = 0; k < GQ_TILES; ++k)
+#pragma unroll
+        for (int i = 0; i < 16; ++i) aQ1[k][i] = 0.f;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) aq1[j] = aQ2[j] = 0.f;
+    const int64_t per = np3 / GP, nchunk = per * B;
+    for (int64_t k = blockIdx.x; k < nchunk; k += gridDim.x) {
+        const int64_t b = k / per, pt = (k - b * per) * GP;
+        __syncthreads();   // the previous chunk has been read
+        for (int c = tid / NZ; c < C; c += GD_T / NZ) sno_cp16(vs + c * GPS + z0, vL + (b * C + c) * np3 + pt + z0);
+        if (tid < NZ) sno_cp16(dys + z0, dy + b * np3 + pt + z0);
+        sno_commit();
+        sno_wait_all();
+        __syncthreads();
+        const float4 dyv = *reinterpret_cast<const float4*>(dys + z0);
+        if (p0 < d.PP) {
+            float a[8][4];
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) a[j][i] = pq[p0 + j];
+            for (int c = 0; c < C; ++c) {
+                const float4 x = *reinterpret_cast<const float4*>(vs + c * GPS + z0);
+                const float4 w0 = *reinterpret_cast<const float4*>(Qt + c * d.PP + p0);
+                const float4 w1 = *reinterpret_cast<const float4*>(Qt + c * d.PP + p0 + 4);
+                const float wv[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    a[j][0] = fmaf(wv[j], x.x, a[j][0]);
+                    a[j][1] = fmaf(wv[j], x.y, a[j][1]);
+                    a[j][2] = fmaf(wv[j], x.z, a[j][2]);
+                    a[j][3] = fmaf(wv[j], x.w, a[j][3]);
                 }
             }
-        }
-        __syncthreads();
-        if (!first) {
-            zfwd_rows(dn, tb, C, n, m, czb + (b * C * n2 + xy) * m, n2 * m);
-            tile_sums<NT_W>(dn, ws, C, C, n, aW);   // dW_{l-1}[o][c] += sum_z dz_{l-1}[o][z] v_{l-1}[c][z]
-        }
-        if (threadIdx.x < C) {
-            float sum = 0.f, s1 = 0.f;
-            for (int zz = 0; zz < n; ++zz) {
-                const float d = dn[threadIdx.x * ns + zz];
-                sum += d;
-                if (first) s1 = fmaf(d, ws[zz], s1);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const float w = pq[d.PP + p0 + j];
+                const float4 g = make_float4(dyv.x * w * gelu_d(a[j][0]), dyv.y * w * gelu_d(a[j][1]),
+                                             dyv.z * w * gelu_d(a[j][2]), dyv.w * w * gelu_d(a[j][3]));
+                aQ2[j] = fmaf(dyv.x, gelu_f(a[j][0]), fmaf(dyv.y, gelu_f(a[j][1]),
+                         fmaf(dyv.z, gelu_f(a[j][2]), fmaf(dyv.w, gelu_f(a[j][3]), aQ2[j]))));
+                aq1[j] += (g.x + g.y) + (g.z + g.w);
+                *reinterpret_cast<float4*>(das + (p0 + j) * GPS + z0) = g;
             }
-            ab += sum;
-            aw1 += s1;
+        }
+        if (tid < NZ) aq2 += (dyv.x + dyv.y) + (dyv.z + dyv.w);
+        __syncthreads();
+        for (int cb = tid / NZ; cb < nt; cb += GD_T / NZ) {   // dz: 4 channels x 4 points
+            float a[4][4] = {};
+            for (int p = 0; p < d.PP; ++p) {
+                const float4 x = *reinterpret_cast<const float4*>(das + p * GPS + z0);
+                const float4 w = *reinterpret_cast<const float4*>(Qs + p * d.C4 + 4 * cb);
+                const float wv[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    a[j][0] = fmaf(wv[j], x.x, a[j][0]);
+                    a[j][1] = fmaf(wv[j], x.y, a[j][1]);
+                    a[j][2] = fmaf(wv[j], x.z, a[j][2]);
+                    a[j][3] = fmaf(wv[j], x.w, a[j][3]);
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                *reinterpret_cast<float4*>(dz + (b * C + 4 * cb + j) * np3 + pt + z0) =
+                    make_float4(a[j][0], a[j][1], a[j][2], a[j][3]);
+        }
+#pragma unroll
+        for (int j = 0; j < GQ_TILES; ++j) {
+            const int t = tid / S + j * (GD_T / S);
+            if (t < tiles) grad_tile(das + 4 * (t / nt) * GPS, vs + 4 * (t % nt) * GPS, s, S, aQ1[j]);
         }
     }
-    if (!first) {
-        tile_flush<NT_W>(aW, C, C, gW);
-        if (threadIdx.x < C) atomicAdd(gb + threadIdx.x, ab);
-    } else if (threadIdx.x < C) {
-        atomicAdd(gWl + threadIdx.x, aw1);
-        atomicAdd(gbl + threadIdx.x, ab);
+#pragma unroll
+    for (int j = 0; j < GQ_TILES; ++j) {
+        const int t = tid / S + j * (GD_T / S);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            const float a = lane_sum(aQ1[j][i], S);
+            const int p = 4 * (t / nt) + i / 4;
+            if (t < tiles && !s && p < P) atomicAdd(gQ1 + p * C + 4 * (t % nt) + i % 4, a);
+        }
     }
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        const float a = lane_sum(aq1[j], NZ), h = lane_sum(aQ2[j], NZ);
+        if (!zb && p0 + j < P) {
+            atomicAdd(gq1 + p0 + j, a);
+            atomicAdd(gQ2 + p0 + j, h);
+        }
+    }
+    aq2 = lane_sum(aq2, NZ);
+    if (tid == 0) atomicAdd(gq2, aq2);
 }
 
 // loss and dL/dy: mean squared error; dy = 2 (y - t) / (B np3)
@@ -1359,7 +1307,7 @@ static int forward(SnoModel& M, const float* u, float* y, int B, bool train) {
         const ZRowDims d = zrow_dims(n, C, m, M.P, last);
         const int rows = B * n * n;
         int per_sm = 1;
-        auto* kz = last ? k_zrow<true> : k_zrow<false>;   // (the last layer's rows go into the projection)
+        auto* kz = last ? k_zrow<ZR_PROJ> : k_zrow<ZR_FWD>;   // (the last layer's rows go into the projection)
         KF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kz, ZF_T, d.smem));
         const int grid = std::min((rows + d.R - 1) / d.R, std::max(1, per_sm) * M.num_sms);
         kz<<<grid, ZF_T, d.smem, st>>>(
@@ -1390,35 +1338,48 @@ static int loss_grad(SnoModel& M, const float* u, const float* t, int B, double*
     const int q = o_q1(M), L = M.L;
     float* dzA = fld(M.dz, 0, per);
     float* dzB = fld(M.dz, 1, per);
-    k_proj_bwd<<<zr_blocks(M, B), ZR_T, M.zr_smem_b, st>>>(
-        fld(M.v, L, per), fld(M.v, L - 1, per), dy, th + M.off[q], th + M.off[q + 1], th + M.off[q + 2], T + M.tzb,
-        dzA, ptr<float2>(M.cz), gr + M.off[q], gr + M.off[q + 1], gr + M.off[q + 2], gr + M.off[q + 3],
-        gr + M.off[o_w(L - 1)], gr + M.off[o_b(L - 1)], B, C, n, m, M.P);
+    const ProjDims pd = proj_dims(C, M.P);
+    const int64_t nchunk = N / GP, rows = BC * n * n;
+    const size_t gsm = (size_t)4 * C * GPS * 4;
+    int pb_sm = 1, gw_sm = 1;
+    KF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pb_sm, k_proj_bwd, GD_T, pd.smem));
+    KF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&gw_sm, k_grad_w, GD_T, gsm));
+    const unsigned npb = (unsigned)std::min<int64_t>(nchunk, (int64_t)std::max(1, pb_sm) * M.num_sms);
+    const unsigned ngw = (unsigned)std::min<int64_t>(nchunk, (int64_t)std::max(1, gw_sm) * M.num_sms);
+    k_proj_bwd<<<npb, GD_T, pd.smem, st>>>(fld(M.v, L, per), dy, th + M.off[q], th + M.off[q + 1], th + M.off[q + 2],
+                                           dzA, gr + M.off[q], gr + M.off[q + 1], gr + M.off[q + 2], gr + M.off[q + 3],
+                                           B, C, M.P, M.np3, pd);
     KF_LAUNCH();
+    k_lift_u<<<nbs(rows, LU), 256, (size_t)(LU * (n / 2 + 1) + n / 2 * (m + 1)) * 8, st>>>(
+        dzA, T + M.tfo, ptr<float2>(M.cz), rows, n, m);
+    KF_LAUNCH();
+    const float wn = 1.f / ((float)M.period * M.period * M.period);
+    const ZRowDims zd = zrow_dims(n, C, m, M.P, false);
+    int zb_sm = 1;
+    KF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&zb_sm, k_zrow<ZR_BWD>, ZF_T, zd.smem));
+    const int zgrid = std::min((B * n * n + zd.R - 1) / zd.R, std::max(1, zb_sm) * M.num_sms);
     for (int l = L - 1; l >= 0; --l) {
-        // spectral adjoint of layer l: dG = Tyf Tyf Tzb dz_l (cz holds Tzb dz_l), dR, dV = R^H dG
+        k_grad_w<<<ngw, GD_T, gsm, st>>>(dzA, fld(M.v, l, per), gr + M.off[o_w(l)], gr + M.off[o_b(l)], B, C, M.np3);
+        KF_LAUNCH();
+        // spectral adjoint of layer l (cz holds the last-axis transform of dz_l): dG, dR, dV = R^H dG
         KF_TRY(plane_fwd(M, ptr<float2>(M.cz), ptr<float2>(M.cy), BC * n, m));
-        KF_TRY(plane_fwd(M, ptr<float2>(M.cy), ptr<float2>(M.g), BC, M2 * m));
+        KF_TRY(plane_fwd(M, ptr<float2>(M.cy), ptr<float2>(M.g), BC, M2 * m, wn));
         const unsigned nb = nbs(M.K, M.mix_mb);
         k_mix_grad<<<nb, 256, M.mixg_smem, st>>>(ptr<float2>(M.g), ptr<float2>(M.Vst) + (int64_t)l * BC * M.K,
                                                  gr + M.off[o_rr(l)], gr + M.off[o_ri(l)], B, C, M.K, M.mix_mb);
         KF_LAUNCH();
         KF_TRY(mix(M, l, ptr<float2>(M.g), ptr<float2>(M.ga), B, 1));
-        KF_TRY(plane_inv(M, ptr<float2>(M.ga), ptr<float2>(M.gx), BC, M2 * m));
+        KF_TRY(plane_inv(M, ptr<float2>(M.ga), ptr<float2>(M.gx), BC, M2 * m, 1.f));
         KF_TRY(plane_inv(M, ptr<float2>(M.gx), ptr<float2>(M.gy), BC * n, m));
-        if (l > 0) {
-            k_zinv_point_bwd<<<zr_blocks(M, B), ZR_T, M.zr_smem_f, st>>>(
-                ptr<float2>(M.gy), dzA, th + M.off[o_w(l)], T + M.tzr, fld(M.z, l - 1, per), fld(M.v, l - 1, per),
-                T + M.tzb, dzB, ptr<float2>(M.cz), gr + M.off[o_w(l - 1)], gr + M.off[o_b(l - 1)], nullptr, nullptr,
-                nullptr, B, C, n, m);
-        } else {
-            k_zinv_point_bwd<<<zr_blocks(M, B), ZR_T, M.zr_smem_f, st>>>(
-                ptr<float2>(M.gy), dzA, th + M.off[o_w(l)], T + M.tzr, nullptr, nullptr, T + M.tzb, nullptr, nullptr,
-                nullptr, nullptr, u, gr + M.off[O_WL], gr + M.off[O_BL], B, C, n, m);
-        }
+        k_zrow<ZR_BWD><<<zgrid, ZF_T, zd.smem, st>>>(
+            ptr<float2>(M.gy), dzA, th + M.off[o_w(l)], nullptr, T + M.tfo, l > 0 ? fld(M.z, l - 1, per) : nullptr, dzB,
+            l > 0 ? ptr<float2>(M.cz) : nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr,
+            B * n * n, C, n, m, M.P, zd);
         KF_LAUNCH();
         std::swap(dzA, dzB);
     }
+    k_grad_lift<<<dim3(nbs(M.np3 / 4, 1024), C), 256, 0, st>>>(dzA, u, gr + M.off[O_WL], gr + M.off[O_BL], B, C, M.np3);
+    KF_LAUNCH();
     if (loss_host) {
         KF_CUDA(cudaMemcpyAsync(loss_host, M.loss.p, 8, cudaMemcpyDeviceToHost, st));
         KF_CUDA(cudaStreamSynchronize(st));
@@ -1769,7 +1730,7 @@ int sno_create(sno_model_t* out, int n, int width, int modes, int layers, int pr
                      2 * proj_width + 4 * n) * f4 + al +
                     ((size_t)4 * width * modes + n * (modes + 1) + modes * (n + 2)) * f8;
         const size_t zp = zf + ((size_t)proj_width * C1 + 4 * n + 2 * proj_width) * f4;
-        M.zr_smem_b = (3 * width * ns + 2 * proj_width * ns + proj_width * C1 + 2 * proj_width + n) * f4 + al +
+        const size_t pb = (3 * width * ns + 2 * proj_width * ns + proj_width * C1 + 2 * proj_width + n) * f4 + al +
                       (size_t)modes * ns * f8;
         const size_t per_mode = (size_t)width * (width + 1 + 2 * max_batch) * f8;
         M.mix_mb = (int)std::max<size_t>(1, std::min<size_t>(16, (96u << 10) / per_mode));
@@ -1779,7 +1740,7 @@ int sno_create(sno_model_t* out, int n, int width, int modes, int layers, int pr
         int dev = 0, optin = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-        const size_t need = std::max({M.zr_smem_f, zp, M.zr_smem_b, M.mix_smem, M.mixg_smem, plane_smem, zr});
+        const size_t need = std::max({M.zr_smem_f, zp, pb, M.mix_smem, M.mixg_smem, plane_smem, zr});
         cudaDeviceGetAttribute(&M.num_sms, cudaDevAttrMultiProcessorCount, dev);
         M.num_sms = std::max(M.num_sms, 1);
         if (optin <= 0 || need > (size_t)optin) {
@@ -1789,9 +1750,9 @@ int sno_create(sno_model_t* out, int n, int width, int modes, int layers, int pr
         }
         const int lim = optin;
         cudaFuncSetAttribute(k_lift_z, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-        cudaFuncSetAttribute(k_zrow<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-        cudaFuncSetAttribute(k_zrow<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-        cudaFuncSetAttribute(k_zinv_point_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+        for (auto* k : {k_zrow<ZR_FWD>, k_zrow<ZR_PROJ>, k_zrow<ZR_BWD>})
+            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+        cudaFuncSetAttribute(k_grad_w, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
         cudaFuncSetAttribute(k_proj_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
         for (auto* k : {k_fold_fwd<4>, k_fold_fwd<5>, k_fold_fwd<6>, k_fold_fwd<7>, k_fold_fwd<8>})
             cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
@@ -1823,14 +1784,12 @@ int sno_create(sno_model_t* out, int n, int width, int modes, int layers, int pr
     if ((rc = dev_alloc(M.rbf, (size_t)layers * 2 * M.K * width * width * 2))) return fail(rc);
     M.tzf = 0;
     M.tyf = M.tzf + (int64_t)modes * n;
-    M.tzb = M.tyf + (int64_t)2 * modes * n;
-    M.tzr = M.tzb + (int64_t)modes * n;
-    M.tfo = M.tzr + (int64_t)n * modes;
+    M.tfo = M.tyf + (int64_t)2 * modes * n;
     M.tph = M.tfo + (int64_t)n / 2 * (modes + 1);
     if ((rc = dev_alloc(M.tabs, (M.tph + modes + 1) * sizeof(float2)))) return fail(rc);
     M.period = n;
-    k_tables<<<nbs(2 * modes * n, 128), 128, 0, M.st>>>(n, n, modes, ptr<float2>(M.tabs), M.tzf, M.tyf, M.tzb,
-                                                          M.tzr, M.tfo, M.tph);
+    k_tables<<<nbs(2 * modes * n, 128), 128, 0, M.st>>>(n, n, modes, ptr<float2>(M.tabs), M.tzf, M.tyf, M.tfo,
+                                                          M.tph);
     if (cudaGetLastError() != cudaSuccess) return fail(KIFMM_ERR_CUDA);
     if ((rc = dev_alloc(M.v, (size_t)(layers + 1) * per * 4))) return fail(rc);
     if ((rc = dev_alloc(M.z, (size_t)layers * per * 4))) return fail(rc);
@@ -1871,8 +1830,8 @@ int sno_set_period(sno_model_t h, int period) {
         return KIFMM_ERR_ARG;
     }
     M.period = period;
-    k_tables<<<nbs(2 * M.m * M.n, 128), 128, 0, M.st>>>(M.n, period, M.m, ptr<float2>(M.tabs), M.tzf, M.tyf, M.tzb,
-                                                          M.tzr, M.tfo, M.tph);
+    k_tables<<<nbs(2 * M.m * M.n, 128), 128, 0, M.st>>>(M.n, period, M.m, ptr<float2>(M.tabs), M.tzf, M.tyf, M.tfo,
+                                                          M.tph);
     KF_LAUNCH();
     KF_CUDA(cudaStreamSynchronize(M.st));
     return KIFMM_OK;
