@@ -947,17 +947,19 @@ __global__ void __launch_bounds__(ZF_T, 3) k_zrow(const float2* __restrict__ gy,
 // blocks walk chunks of GP points with 4 x 4 tiles of the sum in registers; where the tiles are fewer
 // than the threads, the chunk's points are split over 2^k lanes a tile (added by shuffles at the end),
 // and a block adds its sums to the gradient once (the row-by-row form added 16384 times 4 rows' sums).
-constexpr int GP = 64;            // points a chunk (n^3 is a multiple of 64)
-constexpr int GPS = GP + 4;       // a channel's row in shared memory
+constexpr int GP = 64;            // points a chunk (n^3 is a multiple of 64); a row in shared memory has 4 more
+constexpr int GPS = GP + 4;
 constexpr int GD_T = 256;
-__device__ __host__ inline int grad_splits(int tiles) {   // lanes a tile, a power of two up to GP / 4
+__device__ __forceinline__ int grad_splits(int tiles) {   // lanes a tile, a power of two up to GP / 4
     int S = GP / 4;
     while (S > 1 && tiles * S > GD_T) S /= 2;
     return S;
 }
 // acc[4 i + j] += sum over the lane's points of X[i][.] Y[j][.]
+template <int NP>
 __device__ __forceinline__ void grad_tile(const float* X, const float* Y, int s, int S, float* acc) {
-    for (int q = 4 * s; q < GP; q += 4 * S) {
+    constexpr int GPS = NP + 4;
+    for (int q = 4 * s; q < NP; q += 4 * S) {
         float4 x[4], w[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
@@ -1007,7 +1009,7 @@ __global__ void __launch_bounds__(GD_T) k_grad_w(const float* __restrict__ dz, c
         sno_commit();
         const float* X = zsh + (it & 1) * 2 * C * GPS;
         if (t < tiles) {
-            grad_tile(X + i0 * GPS, X + (C + j0) * GPS, s, S, acc);
+            grad_tile<GP>(X + i0 * GPS, X + (C + j0) * GPS, s, S, acc);
             if (j0 == 0)
                 for (int q = 4 * s; q < GP; q += 4 * S)
 #pragma unroll
@@ -1059,34 +1061,38 @@ __global__ void __launch_bounds__(256) k_grad_lift(const float* __restrict__ dv,
 }
 
 // backward of the projection: a = Q1 v_L + q1, h = GELU(a), da = dy Q2 GELU'(a), dz_{L-1} = Q1^T da, and the
-// sums dQ1 = da v_L, dq1 = da, dQ2 = dy h, dq2 = dy over all points. Per chunk of GP points: a in tiles of
+// sums dQ1 = da v_L, dq1 = da, dQ2 = dy h, dq2 = dy over all points. Per chunk of NP points (128 where all
+// threads then have a tile of a, P <= 64 and n a multiple of 8, else 64): a in tiles of
 // 8 rows of Q1 x 4 points a thread, da through shared memory, dz in tiles of 4 channels x 4 points, dQ1 as in
-// k_grad_w. Bound by FP32 issue. Width 16, 64 rows, 4 fields of 64^3: 835 -> 408 us (the row-by-row
-// form with the last layer's dW and transform in it; those take 60 us each apart).
+// k_grad_w. Bound by FP32 issue. Width 16, 64 rows, 4 fields of 64^3: 408 us in
+// chunks of 64 (half the threads without a tile of a), 288 us in chunks of 128; the row-by-row form before, with
+// the last layer's dW and transform (60 us each) in it, 835 us.
 constexpr int GQ_TILES = (MAXP / 4) * (MAXC / 4) / GD_T;   // 4 x 4 tiles of dQ1 a thread, at most
 struct ProjDims {
     int PP, C4;   // rows of Q1 in blocks of 8, row stride of Q1 [p][c]
     size_t smem;
 };
-static ProjDims proj_dims(int C, int P) {
+static ProjDims proj_dims(int C, int P, int np) {
     ProjDims d;
     d.PP = (P + 7) & ~7;
     d.C4 = C + 4;
-    d.smem = ((size_t)C * GPS + (size_t)d.PP * GPS + (size_t)C * d.PP + (size_t)d.PP * d.C4 + 2 * d.PP + GP) * 4;
+    d.smem = ((size_t)(C + d.PP) * (np + 4) + (size_t)C * d.PP + (size_t)d.PP * d.C4 + 2 * d.PP + np) * 4;
     return d;
 }
+template <int NP>
 __global__ void __launch_bounds__(GD_T) k_proj_bwd(const float* __restrict__ vL, const float* __restrict__ dy,
                                                    const float* __restrict__ Q1, const float* __restrict__ q1,
                                                    const float* __restrict__ Q2, float* __restrict__ dz, float* gQ1,
                                                    float* gq1, float* gQ2, float* gq2, int B, int C, int P, int64_t np3,
                                                    ProjDims d) {
+    constexpr int GPS = NP + 4;
     extern __shared__ __align__(16) float zsh[];
     float* vs = zsh;                    // v_L [C][GPS]
     float* das = vs + C * GPS;          // da [PP][GPS]
     float* Qt = das + d.PP * GPS;       // Q1 transposed [C][PP]
     float* Qs = Qt + C * d.PP;          // Q1 [PP][C4]
     float* pq = Qs + d.PP * d.C4;       // q1, Q2 [2][PP]
-    float* dys = pq + 2 * d.PP;         // dy [GP]
+    float* dys = pq + 2 * d.PP;         // dy [NP]
     const int tid = threadIdx.x;
     for (int e = tid; e < d.PP * C; e += GD_T) {
         const int p = e / C, c = e - p * C;
@@ -1098,9 +1104,9 @@ __global__ void __launch_bounds__(GD_T) k_proj_bwd(const float* __restrict__ vL,
         pq[p] = p < P ? q1[p] : 0.f;
         pq[d.PP + p] = p < P ? Q2[p] : 0.f;
     }
-    constexpr int NZ = GP / 4;                  // blocks of 4 points
+    constexpr int NZ = NP / 4;                  // blocks of 4 points
     const int nt = C / 4, tiles = d.PP / 4 * nt, S = grad_splits(tiles), s = tid % S;
-    const int zb = tid % NZ, pb = tid / NZ;     // (PP / 8 <= 16 = GD_T / NZ blocks of 8 rows)
+    const int zb = tid % NZ, pb = tid / NZ;     // (PP / 8 <= GD_T / NZ blocks of 8 rows)
     const int z0 = 4 * zb, p0 = 8 * pb;
     float aQ1[GQ_TILES][16], aq1[8], aQ2[8], aq2 = 0.f;
 #pragma unroll
@@ -1109,9 +1115,9 @@ __global__ void __launch_bounds__(GD_T) k_proj_bwd(const float* __restrict__ vL,
         for (int i = 0; i < 16; ++i) aQ1[k][i] = 0.f;
 #pragma unroll
     for (int j = 0; j < 8; ++j) aq1[j] = aQ2[j] = 0.f;
-    const int64_t per = np3 / GP, nchunk = per * B;
+    const int64_t per = np3 / NP, nchunk = per * B;
     for (int64_t k = blockIdx.x; k < nchunk; k += gridDim.x) {
-        const int64_t b = k / per, pt = (k - b * per) * GP;
+        const int64_t b = k / per, pt = (k - b * per) * NP;
         __syncthreads();   // the previous chunk has been read
         for (int c = tid / NZ; c < C; c += GD_T / NZ) sno_cp16(vs + c * GPS + z0, vL + (b * C + c) * np3 + pt + z0);
         if (tid < NZ) sno_cp16(dys + z0, dy + b * np3 + pt + z0);
@@ -1173,7 +1179,7 @@ __global__ void __launch_bounds__(GD_T) k_proj_bwd(const float* __restrict__ vL,
 #pragma unroll
         for (int j = 0; j < GQ_TILES; ++j) {
             const int t = tid / S + j * (GD_T / S);
-            if (t < tiles) grad_tile(das + 4 * (t / nt) * GPS, vs + 4 * (t % nt) * GPS, s, S, aQ1[j]);
+            if (t < tiles) grad_tile<NP>(das + 4 * (t / nt) * GPS, vs + 4 * (t % nt) * GPS, s, S, aQ1[j]);
         }
     }
 #pragma unroll
@@ -1388,15 +1394,17 @@ static int loss_grad(SnoModel& M, const float* u, const float* t, int B, double*
     const int q = o_q1(M), L = M.L;
     float* dzA = fld(M.dz, 0, per);
     float* dzB = fld(M.dz, 1, per);
-    const ProjDims pd = proj_dims(C, M.P);
+    const bool wide = M.P <= 64 && n % 8 == 0;   // chunks of the projection's backward
+    const ProjDims pd = proj_dims(C, M.P, wide ? 128 : 64);
+    auto* kpb = wide ? k_proj_bwd<128> : k_proj_bwd<64>;
     const int64_t nchunk = N / GP, rows = BC * n * n;
     const size_t gsm = (size_t)4 * C * GPS * 4;
     int pb_sm = 1, gw_sm = 1;
-    KF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pb_sm, k_proj_bwd, GD_T, pd.smem));
+    KF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pb_sm, kpb, GD_T, pd.smem));
     KF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&gw_sm, k_grad_w, GD_T, gsm));
-    const unsigned npb = (unsigned)std::min<int64_t>(nchunk, (int64_t)std::max(1, pb_sm) * M.num_sms);
+    const unsigned npb = (unsigned)std::min<int64_t>(N / (wide ? 128 : 64), (int64_t)std::max(1, pb_sm) * M.num_sms);
     const unsigned ngw = (unsigned)std::min<int64_t>(nchunk, (int64_t)std::max(1, gw_sm) * M.num_sms);
-    k_proj_bwd<<<npb, GD_T, pd.smem, st>>>(fld(M.v, L, per), dy, th + M.off[q], th + M.off[q + 1], th + M.off[q + 2],
+    kpb<<<npb, GD_T, pd.smem, st>>>(fld(M.v, L, per), dy, th + M.off[q], th + M.off[q + 1], th + M.off[q + 2],
                                            dzA, gr + M.off[q], gr + M.off[q + 1], gr + M.off[q + 2], gr + M.off[q + 3],
                                            B, C, M.P, M.np3, pd);
     KF_LAUNCH();
@@ -1803,7 +1811,8 @@ int sno_create(sno_model_t* out, int n, int width, int modes, int layers, int pr
         for (auto* k : {k_zrow<ZR_FWD>, k_zrow<ZR_PROJ>, k_zrow<ZR_BWD>})
             cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
         cudaFuncSetAttribute(k_grad_w, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-        cudaFuncSetAttribute(k_proj_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+        cudaFuncSetAttribute(k_proj_bwd<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+        cudaFuncSetAttribute(k_proj_bwd<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
         for (auto* k : {k_fold_fwd<4>, k_fold_fwd<5>, k_fold_fwd<6>, k_fold_fwd<7>, k_fold_fwd<8>})
             cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
         cudaFuncSetAttribute(k_fold_inv, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
