@@ -62,7 +62,7 @@ static void free_plan(Plan* p) {
                       &p->q, &p->Isort, &p->chk, &p->chkx, &p->cu, &p->cu32, &p->chl, &p->cexp, &p->ozBox, &p->ozEb, &p->dd, &p->phid, &p->phiu,
                       &p->far, &p->wleaves, &p->host_I, &p->host_S, &p->err,
                       &p->tc_tiles, &p->tc_boxes, &p->tc_slots, &p->ptab, &p->l2l_slots, &p->m2m_tiles, &p->m2m_slots, &p->stage32, &p->m2m_chl, &p->apply_part, &p->nf_utab, &p->nf_Ttc, &p->nf_tiles,
-                      &p->nf_slots, &p->nf_boxes, &p->nf_qhl, &p->nf_qexp, &p->nf_near, &p->lat_P, &p->lat_Q, &p->lat_Ttc, &p->lat_iota, &p->lat_slots, &p->lat_fst, &p->lat_Mimg, &p->lat_Mer, &p->nf_ref})
+                      &p->nf_slots, &p->nf_boxes, &p->nf_qhl, &p->nf_qexp, &p->nf_near, &p->p2p_near, &p->lat_P, &p->lat_Q, &p->lat_Ttc, &p->lat_iota, &p->lat_slots, &p->lat_fst, &p->lat_Mimg, &p->lat_Mer, &p->nf_ref})
         dev_free(*b);
     auto free_sched = [](TcSched& s) {
         for (DevBuf* b : {&s.pre, &s.first, &s.src, &s.meta, &s.part}) dev_free(*b);

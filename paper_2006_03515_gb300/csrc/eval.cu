@@ -528,6 +528,7 @@ int build_eval_data(Plan& p) {
     dev_free(flag); dev_free(pos); dev_free(scan_tmp);
     if (p.precision == KIFMM_MIXED) KF_TRY(p2p_series_check(p));
     KF_TRY(near_tc_plan(p));
+    KF_TRY(p2p_fork_plan(p));
     // FP64-exact upward solves on the tensor cores (mixed form; KIFMM_UPWARD=fp64 keeps the FP64 pipe)
     {
         const char* up = std::getenv("KIFMM_UPWARD");
@@ -1642,7 +1643,7 @@ template <bool SERIES, class TO>
 __global__ void __launch_bounds__(P2Q_T) k_p2p_mixed(EvalView E, const int32_t* leaves, const int32_t* uoff,
                                                      const int32_t* uitems, const double* q, const double* far,
                                                      const double* sigma, const double* Is, const int32_t* perm,
-                                                     double C, TO* out) {
+                                                     double C, TO* out, double* near) {
     const int B = leaves[blockIdx.x];
     const double* cB = E.centre + 3 * (int64_t)B;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1726,11 +1727,19 @@ __global__ void __launch_bounds__(P2Q_T) k_p2p_mixed(EvalView E, const int32_t* 
             if (i < p1) {
                 double s = 0;
                 for (int k = 0; k < P2Q_GRP; ++k) s += red[k][tl];
-                if (perm[i] < E.n_real) out[perm[i]] = (TO)(C * (s + far[i] + sigma[i] * Is[i]));
+                if (near) near[i] = s;   // (beside the far field: k_p2p_finish adds them)
+                else if (perm[i] < E.n_real) out[perm[i]] = (TO)(C * (s + far[i] + sigma[i] * Is[i]));
             }
         }
         __syncthreads();
     }
+}
+template <class TO>
+__global__ void __launch_bounds__(256) k_p2p_finish(const double* near, const double* far, const double* sigma,
+                                                    const double* Is, const int32_t* perm, int64_t n, int64_t n_real,
+                                                    double C, TO* out) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n && perm[i] < n_real) out[perm[i]] = (TO)(C * (near[i] + far[i] + sigma[i] * Is[i]));
 }
 
 // Plan time: the smallest squared distance (box-local FP32 coordinates, as in the pair
@@ -1871,6 +1880,38 @@ static int launch_apply(cudaStream_t st, const T* Op, int ldop, int Mo, int Ki, 
 // the near sums on the plan's second stream, after the work ordered before near_ev[0] on the
 // plan's stream; near_ev[1] is recorded whatever happened, so that a join never waits on an
 // unrecorded event and a capture never holds an open fork
+// the generic pair sums into p2p_near, on stream st (they read only the sorted weights)
+static int near_pairs(Plan& p, cudaStream_t st, int64_t& nl) {
+    auto* k = p.p2p_series ? k_p2p_mixed<true, float> : k_p2p_mixed<false, float>;
+    k<<<(unsigned)p.nleaves, P2Q_T, (size_t)P2Q_CHUNK * 16, st>>>(
+        make_view(p), ptr<int32_t>(p.leaves), ptr<int32_t>(p.lists[0].off), ptr<int32_t>(p.lists[0].items),
+        ptr<double>(p.q), nullptr, nullptr, nullptr, nullptr, 0.0, nullptr, ptr<double>(p.p2p_near));
+    KF_LAUNCH();
+    ++nl;
+    return KIFMM_OK;
+}
+
+// The generic pair sums (plans off the lattice) read only the sorted weights as well: issued after the M2L
+// on the second stream, they fill what its last wave and the small levels of the downward pass leave idle
+// (not the M2L itself: its stages take the whole shared memory of an SM). Evaluations without and with:
+// refined grid of 1632 leaves 1215 -> 1135 us, 60 x 52 x 44 cells 522 -> 499 us, 96 x 90 x 100 cells 2828 ->
+// 2808 us, two-level grid of 3.2 M cells 7437 -> 7419 us. Fewer leaves than these were not measured and keep
+// one stream.
+constexpr int64_t P2P_FORK_LEAVES = 1024;
+int p2p_fork_plan(Plan& p) {
+    const char* ns = std::getenv("KIFMM_NEAR_STREAM");
+    if (p.precision != KIFMM_MIXED || p.near_tc || !p.m2l_tensor || p.tree.nlevels <= 2 ||
+        p.nleaves < P2P_FORK_LEAVES || (ns && std::string(ns) == "same"))
+        return KIFMM_OK;
+    KF_TRY(dev_alloc(p.p2p_near, (size_t)p.tree.n * 8));
+    if (!p.near_st) {
+        KF_CUDA(cudaStreamCreateWithFlags(&p.near_st, cudaStreamNonBlocking));
+        for (auto& e : p.near_ev) KF_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    }
+    p.p2p_fork = true;
+    return KIFMM_OK;
+}
+
 static int near_fork_launch(Plan& p, int64_t& nl) {
     cudaError_t e = cudaStreamWaitEvent(p.near_st, p.near_ev[0], 0);
     int rc = KIFMM_OK;
@@ -1881,7 +1922,7 @@ static int near_fork_launch(Plan& p, int64_t& nl) {
     p.near_forked = true;
     p.near_pending = false;
     if (p.timing && p.near_tev[0]) cudaEventRecord(p.near_tev[0], p.near_st);
-    rc = near_tc_contract(p, p.near_st, nl);
+    rc = p.near_tc ? near_tc_contract(p, p.near_st, nl) : near_pairs(p, p.near_st, nl);
     if (p.timing && p.near_tev[1]) cudaEventRecord(p.near_tev[1], p.near_st);
     e = cudaEventRecord(p.near_ev[1], p.near_st);
     if (rc == KIFMM_OK && e != cudaSuccess) {
@@ -2149,7 +2190,7 @@ int run_eval(Plan& p, const void* I, void* S_out, int dtype, double C) {
     // the M2L starts (the far field's run_far issues them after its M2L launch), so that the
     // earlier-issued M2L takes the SMs first and the near sums fill its last wave and the
     // downward pass; without a far field, right here.
-    const bool fork = mixed && p.near_tc && p.near_st;
+    const bool fork = mixed && p.near_st && (p.near_tc || p.p2p_fork);
     p.near_forked = false;
     p.near_pending = fork && t.nlevels > 2 && !p.near_fork_early;
     if (fork && !p.near_pending) {
@@ -2223,6 +2264,18 @@ int run_eval(Plan& p, const void* I, void* S_out, int dtype, double C) {
         if (p.near_forked) KF_CUDA(cudaStreamWaitEvent(st, p.near_ev[1], 0));   // join
         else KF_TRY(near_tc_contract(p, st, nl));
         KF_TRY(near_tc_finish(p, ptr<double>(p.far), C, S_out, dtype, nl));
+    } else if (p.near_forked) {   // the pair sums ran beside the far field
+        KF_CUDA(cudaStreamWaitEvent(st, p.near_ev[1], 0));
+        if (dtype == KIFMM_F64)
+            k_p2p_finish<double><<<nbk(n, 256), 256, 0, st>>>(ptr<double>(p.p2p_near), ptr<double>(p.far), ptr<double>(p.sigma),
+                                                              ptr<double>(p.Isort), ptr<int32_t>(t.perm), n, E.n_real, C,
+                                                              (double*)S_out);
+        else
+            k_p2p_finish<float><<<nbk(n, 256), 256, 0, st>>>(ptr<double>(p.p2p_near), ptr<double>(p.far), ptr<double>(p.sigma),
+                                                             ptr<double>(p.Isort), ptr<int32_t>(t.perm), n, E.n_real, C,
+                                                             (float*)S_out);
+        KF_LAUNCH();
+        ++nl;
     } else {
         size_t smem = (size_t)(mixed ? P2Q_CHUNK : P2P_CHUNK) * 16;
         const int32_t* uo = ptr<int32_t>(p.lists[0].off);
@@ -2234,11 +2287,11 @@ int run_eval(Plan& p, const void* I, void* S_out, int dtype, double C) {
             if (dtype == KIFMM_F64)
                 kf64<<<g, P2Q_T, smem, st>>>(E, ptr<int32_t>(p.leaves), uo, ui, ptr<double>(p.q), ptr<double>(p.far),
                                              ptr<double>(p.sigma), ptr<double>(p.Isort), ptr<int32_t>(t.perm), C,
-                                             (double*)S_out);
+                                             (double*)S_out, nullptr);
             else
                 kf32<<<g, P2Q_T, smem, st>>>(E, ptr<int32_t>(p.leaves), uo, ui, ptr<double>(p.q), ptr<double>(p.far),
                                              ptr<double>(p.sigma), ptr<double>(p.Isort), ptr<int32_t>(t.perm), C,
-                                             (float*)S_out);
+                                             (float*)S_out, nullptr);
         } else {
             if (dtype == KIFMM_F64)
                 k_p2p<false, double><<<g, P2P_T, smem, st>>>(E, ptr<int32_t>(p.leaves), uo, ui, ptr<double>(p.q), ptr<double>(p.far),

@@ -260,6 +260,8 @@ struct Plan {
     std::vector<cudaEvent_t> lane_ev;
     // the near-field contraction's own stream (tensor-core lattice near field): it needs only
     // the sorted weights, so it runs beside the far field; events [0] fork, [1] join
+    DevBuf p2p_near;             // generic pair sums of every point, when they run on near_st
+    bool p2p_fork = false;       // they do (plans off the lattice with leaves enough)
     cudaStream_t near_st = nullptr;
     cudaEvent_t near_ev[2] = {nullptr, nullptr};
     cudaEvent_t near_tev[2] = {nullptr, nullptr};   // its start and end (phase timing)
@@ -312,6 +314,7 @@ int fft_m2l_plan(Plan& p);
 int fft_m2l_apply(Plan& p, int64_t& nl);
 // near_tc.cu: near field on a uniform lattice
 int near_tc_plan(Plan& p);
+int p2p_fork_plan(Plan& p);   // after near_tc_plan: the generic pair sums' stream and buffer
 int near_tc_contract(Plan& p, cudaStream_t st, int64_t& nl);   // the near sums into nf_near on st
 int near_tc_finish(Plan& p, const double* far, double C, void* out, int dtype, int64_t& nl);
 int lat_s2m(Plan& p);   // chk of every leaf (lat_far plans)
