@@ -493,8 +493,10 @@ static MixDims mix_dims(int C, int B) {
     MixDims d;
     d.BT = std::min(MIX_B, (B + 3) & ~3);
     d.BS = d.BT + 2;
-    d.MB = std::max(1, std::min(16, 256 / ((C / 4) * (d.BT / 4))));   // one item a thread (at most 128 a mode)
-    d.smem = ((size_t)d.MB * C * (C + 2) + (size_t)d.MB * (C * d.BS + 8)) * sizeof(float2);
+    const size_t per = ((size_t)C * (C + 2) + C * d.BS + 8) * sizeof(float2);   // (52 KB at C = 64 and 32 fields)
+    // one item a thread (at most 128 a mode), two blocks an SM
+    d.MB = (int)std::max<size_t>(1, std::min<size_t>({16, (size_t)(256 / ((C / 4) * (d.BT / 4))), (96u << 10) / per}));
+    d.smem = d.MB * per;
     return d;
 }
 template <class TR>

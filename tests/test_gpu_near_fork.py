@@ -7,7 +7,7 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("dims", [(44, 40, 36), (60, 52, 48), (72, 60, 52)])
+@pytest.mark.parametrize("dims", [(28, 24, 20), (44, 40, 36), (60, 52, 48), (72, 60, 52)])
 def test_same_bits_as_on_one_stream(kf, monkeypatch, dims):
     import torch
     h = 1.0 / max(dims)

@@ -19,6 +19,7 @@ SIZES = [   # n, period, width, modes, layers, projection, batch
     (4, 4, 4, 1, 1, 1, 1), (4, 6, 4, 2, 2, 3, 3), (12, 12, 8, 6, 2, 8, 2), (12, 17, 4, 5, 2, 5, 2),
     (20, 30, 4, 7, 2, 16, 1), (24, 24, 8, 8, 1, 8, 1), (28, 42, 4, 9, 1, 7, 1), (40, 60, 12, 3, 2, 16, 2),
     (44, 44, 4, 11, 1, 8, 1), (64, 96, 16, 4, 2, 16, 1),
+    (8, 8, 64, 2, 1, 8, 1), (8, 12, 48, 4, 1, 128, 5),   # wide layers, where a block's modes are few
 ]
 
 
