@@ -62,6 +62,7 @@
 #include <vector>
 
 #include "internal.cuh"
+#include "tc_split.h"
 #include "tcgen05.cuh"
 
 namespace kifmm {
@@ -150,10 +151,6 @@ __global__ void __launch_bounds__(128) k_tc_sources(const int4* tiles, const int
 // ------------------------------------------------------------------------------------
 // the kernel
 // ------------------------------------------------------------------------------------
-// first slot of CTA c's range, and the CTA whose range holds slot g (T slots over n CTAs)
-__host__ __device__ __forceinline__ int tc_range(int c, int T, int n) { return (int)((int64_t)c * T / n); }
-__host__ __device__ __forceinline__ int tc_cta_of(int g, int T, int n) { return (int)((((int64_t)g + 1) * n - 1) / T); }
-
 // R = NB NT coefficients per box; each CTA computes the NT = 32 NC output rows
 // n0 = blockIdx.y NT .. of its tiles (NB > 1 where R exceeds the MMA's N of 256).
 template <int NC, int NS, int NB>
@@ -415,7 +412,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             }
             if (!ok || box < 0) continue;
             const bool cut = p0 < g0 || p1 > g1;   // a piece of the tile: into the work space
-            float4* o = cut ? reinterpret_cast<float4*>(part + ((int64_t)(2 * cta + (p0 < g0 ? 0 : 1)) * TC_M + row) * R + n0 + col0)
+            float4* o = cut ? reinterpret_cast<float4*>(part + ((int64_t)tc_piece(cta, p0, T, ncta) * TC_M + row) * R + n0 + col0)
                             : reinterpret_cast<float4*>(d + (int64_t)box * R + n0 + col0);
 #pragma unroll
             for (int k = 0; k < NT / 8; ++k) {
@@ -453,8 +450,7 @@ __global__ void __launch_bounds__(256) k_tc_finish(const int4* __restrict__ tile
         float4 u[8];
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
-            const int piece = 2 * (c + q) + (tc_range(c + q, T, ncta) > p0 ? 0 : 1);
-            u[q] = c + q <= c1 ? reinterpret_cast<const float4*>(part + ((int64_t)piece * TC_M + row) * R)[col]
+            u[q] = c + q <= c1 ? reinterpret_cast<const float4*>(part + ((int64_t)tc_piece(c + q, p0, T, ncta) * TC_M + row) * R)[col]
                                : make_float4(0.f, 0.f, 0.f, 0.f);
         }
 #pragma unroll
@@ -539,11 +535,6 @@ int m2l_tc_split_f32(cudaStream_t st, const float* c, int64_t nb, int R, void* o
     return KIFMM_OK;
 }
 
-// A tile is cut into pieces of at least this many slots: the start of a CTA (tensor memory, first
-// copies) and the addition of a piece cost about three (32^3, 1250 slots: M2L and addition 76 us
-// with pieces of 6 slots, 34 us with 12).
-constexpr int kTcMinSlots = 12;
-
 int tc_sched_build(cudaStream_t st, const int4* tiles, const int32_t* boxes, const int32_t* vtab, int vstride,
                    const int32_t* slots, int ntiles, int R, int num_sms, TcSched& s) {
     s.ntiles = ntiles;
@@ -563,7 +554,7 @@ int tc_sched_build(cudaStream_t st, const int4* tiles, const int32_t* boxes, con
         pre[k + 1] = (int32_t)sum;
     }
     const int T = s.total = (int)sum;
-    s.ncta = std::max(1, std::min(num_sms / row_blocks(R), std::max(ntiles, T / kTcMinSlots)));
+    s.ncta = tc_num_ctas(T, ntiles, num_sms / row_blocks(R));
     bool cut = false;
     std::vector<int32_t> first(s.ncta, 0);   // each CTA's first tile
     for (int k = 0; k < ntiles; ++k) {
