@@ -82,10 +82,12 @@ __device__ __forceinline__ double exp_neg64(double x, const Pair64Tab& tab) {
     return __double2hiint(X) > __double2hiint(690.0) ? 0.0 : fma(s, p, s);
 }
 
-// e^{-aR} - e^{-bR} times norm / R^3; r2 > 0
+// e^{-aR} - e^{-bR} times norm / R^3; r2 > 0, 0 for an infinite r2 (taken as 2^996)
 __device__ __forceinline__ double pair64_kernel(double r2, const Pair64& k, const Pair64Tab& tab) {
     constexpr double L = 0.69314718055994530942 / kPairTab;   // ln2 / 256
     constexpr double MAGIC = 6755399441055744.0;              // 1.5 2^52: x + MAGIC holds rint(x) in its low word
+    const int r2h = __double2hiint(r2);
+    r2 = __hiloint2double(r2h == 0x7ff00000 ? 0x7e300000 : r2h, __double2loint(r2));
     const double y = rsqrt64(r2);
     const double R = r2 * y;
     // e^{-aR} = s (1 + p): s = 2^{-ka/256}
