@@ -125,6 +125,12 @@ void kifmm_default_opts(kifmm_opts* o) {
 
 const char* kifmm_last_error(void) { return g_last_error.c_str(); }
 
+// A plan of checked arguments. no_fft: without the transforms of the FP64 form's M2L; *took_fft: whether a plan
+// that failed had taken them.
+static int make_plan(kifmm_plan_t* out, const double* points, int64_t n, const double* cell_h, double uniform_h,
+                     int leaf_size, int surface_order, double a, double b, kifmm_opts o, bool rect, bool no_fft,
+                     bool* took_fft);
+
 int kifmm_plan(kifmm_plan_t* out, const double* points, int64_t n, const double* cell_h, double uniform_h,
                int leaf_size, int surface_order, double a, double b, const kifmm_opts* opts_in) {
     set_error("");
@@ -205,11 +211,24 @@ int kifmm_plan(kifmm_plan_t* out, const double* points, int64_t n, const double*
         return KIFMM_ERR_ARG;
     }
     AllocFaultScope fault_scope;
+    bool took_fft = false;
+    int rc = make_plan(out, points, n, cell_h, uniform_h, leaf_size, surface_order, a, b, o, rect, false, &took_fft);
+    if (rc == KIFMM_ERR_OOM && took_fft) {   // the dense products' memory does not grow with the boxes
+        set_error("");
+        rc = make_plan(out, points, n, cell_h, uniform_h, leaf_size, surface_order, a, b, o, rect, true, &took_fft);
+    }
+    return rc;
+}
+
+static int make_plan(kifmm_plan_t* out, const double* points, int64_t n, const double* cell_h, double uniform_h,
+                     int leaf_size, int surface_order, double a, double b, kifmm_opts o, bool rect, bool no_fft,
+                     bool* took_fft) {
     Plan* p = new (std::nothrow) Plan();
     if (!p) {
         set_error("kifmm_plan: host allocation failed");
         return KIFMM_ERR_OOM;
     }
+    p->no_fft = no_fft;
     p->precision = o.precision;
     p->self_mode = o.self_mode;
     p->kind = o.kernel;
@@ -233,6 +252,7 @@ int kifmm_plan(kifmm_plan_t* out, const double* points, int64_t n, const double*
     for (int k = 0; k < 3; ++k) p->cell_dims[k] = p->rect ? o.cell_dims[k] : 0.0;
     auto fail = [&](int rc) {
         std::string msg = g_last_error;
+        *took_fft = p->fft_m2l;
         free_plan(p);
         cudaGetLastError();
         g_last_error = msg;

@@ -213,6 +213,7 @@ int build_eval_data(Plan& p) {
     KF_LAUNCH();
 
     DevBuf flag, pos, scan_tmp;
+    DevTemps temps{{&flag, &pos, &scan_tmp}};
     KF_TRY(dev_alloc(flag, (nb + 1) * 4));
     KF_TRY(dev_alloc(pos, (nb + 1) * 4));
     // all leaves, and leaves of level >= 2 (P2M)

@@ -205,16 +205,28 @@ __global__ void __launch_bounds__(FF_T) k_fft_m2l(int m0, int S, int64_t b0, con
     }
 }
 
-// The FP64 form of the surface representation takes the transforms up to m0 = 8 (beyond, a table
-// transform's scratch leaves shared memory) while the spectra stay below 16 GB; KIFMM_M2L=simt keeps the
-// dense products.
+// The FP64 form of the surface representation takes the transforms up to m0 = 8 (the evaluation's kernels
+// then stay within 48 KB of shared memory), where their memory, which grows with the boxes (12.8 KB each at
+// m0 = 6), is no more than that of the dense products' tables (45 MB a level), or else at most 16 GB of spectra
+// and an eighth of what the device has free, so that plans made side by side do not crowd out one another; a plan that
+// still runs out of memory is made again without them (kifmm_plan). KIFMM_M2L=simt keeps the dense products.
 bool fft_m2l_wanted(const Plan& p) {
     const char* m2l = std::getenv("KIFMM_M2L");
-    if (p.precision != KIFMM_FP64 || p.cheb || p.m0 > FF_MAXM0 || (m2l && std::string(m2l) == "simt")) return false;
-    return (double)p.tree.nboxes * ff_nf(p.m0) * 16.0 <= 16e9;
+    if (p.precision != KIFMM_FP64 || p.cheb || p.m0 > FF_MAXM0 || p.no_fft || (m2l && std::string(m2l) == "simt"))
+        return false;
+    const double nf = ff_nf(p.m0), slots = (double)(p.tree.nlevels - 2) * kOffsetSlots, spec = p.tree.nboxes * nf * 16.0;
+    const double need = spec + p.tree.nboxes * p.S * 8.0 + slots * nf * 16.0;
+    if (need <= slots * p.R * p.R * 8.0) return true;
+    size_t free_b = 0, total_b = 0;
+    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return spec <= 16e9 && need <= free_b / 8.0;
 }
 
 int fft_m2l_plan(Plan& p) {
+    p.fft_m2l = true;
     cudaStream_t st = p.stream;
     const int m0 = p.m0, nf = ff_nf(m0), n = 2 * m0 - 1, L = p.tree.nlevels;
     std::vector<int32_t> lidx((size_t)m0 * m0 * m0, -1);
@@ -241,7 +253,6 @@ int fft_m2l_plan(Plan& p) {
         KF_LAUNCH();
     }
     KF_CUDA(cudaStreamSynchronize(st));
-    p.fft_m2l = true;
     return KIFMM_OK;
 }
 

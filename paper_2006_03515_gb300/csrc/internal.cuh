@@ -68,6 +68,13 @@ struct AllocFaultScope {
     ~AllocFaultScope();
 };
 void dev_free(DevBuf& b);
+// frees a function's own buffers on every way out of it
+struct DevTemps {
+    std::vector<DevBuf*> bufs;
+    ~DevTemps() {
+        for (DevBuf* b : bufs) dev_free(*b);
+    }
+};
 template <class T> T* ptr(const DevBuf& b) { return reinterpret_cast<T*>(b.p); }
 
 // Split of one tensor-core translation launch over the SMs (m2l_tc.cu): prefix sums of the tiles'
@@ -238,6 +245,7 @@ struct Plan {
     DevBuf tc_slots;             // [tile][344] active offset slots
     int tc_ntiles = 0;
     bool fft_m2l = false;        // FP64 form: M2L by Fourier transforms (fft_m2l.cu)
+    bool no_fft = false;         // not by them (the device's memory did not hold them)
     DevBuf fft_idx, fft_tab, fft_spec, fft_q;   // lattice point -> surface point; [level - 2][343] kernel
                                                 // transforms; box spectra; [box][S] densities, then potentials
     TcSched sch_m2l, sch_near, sch_lat, sch_l2l[kMaxLevel + 1], sch_m2m[kMaxLevel + 1];

@@ -395,7 +395,8 @@ int build_operators(Plan& p) {
 
     const int nlev = L - 2;        // levels 2 .. L-1
     const int64_t SS = (int64_t)S * S;
-    DevBuf A, V, sig, rank, conv, shifts, tmp, z, idxb;
+    DevBuf A, V, sig, rank, conv, shifts, tmp, z, idxb, m2l, w;
+    DevTemps temps{{&A, &V, &sig, &rank, &conv, &shifts, &tmp, &z, &idxb, &m2l, &w}};
     KF_TRY(dev_alloc(A, nlev * SS * 8));
     KF_TRY(dev_alloc(V, nlev * SS * 8));
     KF_TRY(dev_alloc(sig, nlev * S * 8));
@@ -470,7 +471,6 @@ int build_operators(Plan& p) {
         KF_CUDA(cudaStreamSynchronize(st));   // idxb is reused by the next level
     }
     // ---- M2L in coefficients: T_{l,delta} = V^T K(x^{B,d}, y^{A,u}) V, c_A - c_B = 2 r delta
-    DevBuf m2l, w;
     KF_TRY(dev_alloc(m2l, kOffsetSlots * SS * 8));
     KF_TRY(dev_alloc(w, kOffsetSlots * SR * 8));
     std::vector<double> sh(kOffsetSlots * 3);
@@ -554,7 +554,6 @@ int build_operators(Plan& p) {
         }
     }
     KF_CUDA(cudaStreamSynchronize(st));
-    for (DevBuf* d : {&A, &V, &sig, &rank, &conv, &shifts, &tmp, &z, &idxb, &m2l, &w}) dev_free(*d);
     return KIFMM_OK;
 }
 
@@ -633,7 +632,8 @@ int build_self_terms(Plan& p, const double* h_dev, double uh) {
     cudaStream_t st = p.stream;
     const int64_t n = p.tree.n;
     const int NQ = 64;
-    DevBuf gx, gw;
+    DevBuf gx, gw, hb, sb, key, val, tk, tv, hist, flag, pos, scan_tmp, hs, su;
+    DevTemps temps{{&gx, &gw, &hb, &sb, &key, &val, &tk, &tv, &hist, &flag, &pos, &scan_tmp, &hs, &su}};
     KF_TRY(dev_alloc(gx, NQ * 8));
     KF_TRY(dev_alloc(gw, NQ * 8));
     gauss_legendre<<<1, NQ, 0, st>>>(NQ, ptr<double>(gx), ptr<double>(gw));
@@ -641,7 +641,6 @@ int build_self_terms(Plan& p, const double* h_dev, double uh) {
     KF_TRY(dev_alloc(p.sigma, n * 8));
     KF_TRY(dev_alloc(p.w, n * 8));
     if (!h_dev) {   // one cell shape for every point: a cube of edge uh, or the plan's rectangular cell
-        DevBuf hb, sb;
         KF_TRY(dev_alloc(hb, 8));
         KF_TRY(dev_alloc(sb, 8));
         KF_CUDA(cudaMemcpyAsync(hb.p, &uh, 8, cudaMemcpyHostToDevice, st));
@@ -667,10 +666,8 @@ int build_self_terms(Plan& p, const double* h_dev, double uh) {
         fill_uniform<<<nb(n, 256), 256, 0, st>>>(n, s, vol, ptr<double>(p.sigma), ptr<double>(p.w));
         KF_LAUNCH();
         KF_CUDA(cudaStreamSynchronize(st));
-        dev_free(hb); dev_free(sb); dev_free(gx); dev_free(gw);
         return KIFMM_OK;
     }
-    DevBuf key, val, tk, tv, hist, flag, pos, scan_tmp, hs, su;
     KF_TRY(dev_alloc(key, n * 8));
     KF_TRY(dev_alloc(val, n * 4));
     KF_TRY(dev_alloc(flag, n * 4));
@@ -699,7 +696,6 @@ int build_self_terms(Plan& p, const double* h_dev, double uh) {
                                               ptr<double>(p.w));
     KF_LAUNCH();
     KF_CUDA(cudaStreamSynchronize(st));
-    for (DevBuf* d : {&key, &val, &tk, &tv, &hist, &flag, &pos, &scan_tmp, &hs, &su, &gx, &gw}) dev_free(*d);
     return KIFMM_OK;
 }
 
