@@ -610,14 +610,18 @@ int kifmm_get_info(kifmm_plan_t h, kifmm_info* info) {
     info->m2l_tensor = p.m2l_tensor ? 1 : 0;
     info->near_tensor = p.near_tc ? 1 : 0;
     info->lattice_far = p.lat_far ? 1 : 0;
-    {   // the same conditions as the evaluation's dispatch of M2M, L2L and the upward solves
+    // levels whose upward solve runs as exact slices (the evaluation's dispatch)
+    auto up_tensor = [&p](int l) {
+        return !p.cheb && ((p.lat_up && l == p.nf_level) || (p.oz && p.lv[l].n_up > p.oz_min));
+    };
+    {   // the same conditions as the evaluation's dispatch of M2M and L2L
         const bool mixed = p.precision == KIFMM_MIXED;
         int64_t nm = 0, nl2 = 0, nup = 0;
         for (int l = 2; l < p.tree.nlevels; ++l) {
             if (p.lv[l].n_par > 0 && mixed && !p.cheb && p.m2m_tc && p.m2m_count[l] >= p.tc_min_tiles) ++nm;
             if (l >= 3 && p.lv[l - 1].l2l_max > 0 && mixed && !p.cheb && p.l2l_tc && p.tc_count[l] >= p.tc_min_tiles)
                 ++nl2;
-            if (!p.cheb && ((p.lat_up && l == p.nf_level) || (p.oz && p.lv[l].n_up > p.oz_min))) ++nup;
+            if (up_tensor(l)) ++nup;
         }
         info->m2m_tensor_levels = nm;
         info->l2l_tensor_levels = nl2;
@@ -633,10 +637,9 @@ int kifmm_get_info(kifmm_plan_t h, kifmm_info* info) {
                 up += 2.0 * p.ops[l].rank * (p.lat_up && l == p.nf_level ? p.nf_R : p.S) * p.lv[l].n_up;
         info->upward_flops = up;
         double mma = 0;
-        if (p.oz)
-            for (int l = 2; l < p.tree.nlevels; ++l)
-                if (p.lv[l].n_up > p.oz_min)
-                    mma += pinv_oz_mma_flops(p.lat_up && l == p.nf_level ? p.nf_R : p.S, p.ops[l].rank, p.lv[l].n_up);
+        for (int l = 2; l < p.tree.nlevels; ++l)
+            if (up_tensor(l))
+                mma += pinv_oz_mma_flops(p.lat_up && l == p.nf_level ? p.nf_R : p.S, p.ops[l].rank, p.lv[l].n_up);
         info->upward_mma_flops = mma;
     }
     info->device_error = 0;
