@@ -33,8 +33,8 @@
 //  * PW producer warps: eight lanes copy one source row's 128-byte piece with 16-byte cp.async
 //    (zero-filled where the box has no source at this offset), so a warp instruction touches four
 //    lines; with a row per lane it touched 32. Thread 0 also moves the pre-swizzled B chunk with one
-//    1-D bulk copy. A warp reports a stage on its "full" mbarrier once its own copies of it have
-//    arrived: while it waits for a free stage it reports the pending ones, oldest first.
+//    1-D bulk copy. A thread's arrival on the stage's "full" mbarrier is left to the hardware, when its
+//    copies are there (cp.async.mbarrier.arrive.noinc), so it goes on to the next free stage at once.
 //  * MMA warp, lane 0: waits for a full stage, issues its k-steps x 3 MMAs into the slot's two
 //    tensor-memory accumulators (hi x hi terms; cross terms) and commits the stage's "empty"
 //    mbarrier; after the last chunk of a slot it commits the accumulators' "ready" mbarrier. MMAs are
@@ -52,7 +52,8 @@
 // (R = 128) 985 -> 599 us, one wave of the chip at 64^3 506 -> 92 us, 1250 slots in five tiles at 32^3
 // 507 -> 25 us, the near field's 6912 slots at 128^3 (R = 64) 78 -> 50 us. At 128^3 the tensor pipe is
 // active half of the time; the MMA thread's waits and proxy fences take most of the rest.
-// Every wait is bounded; a timeout sets an abort flag that ends the other roles' waits,
+// Every wait is bounded; a timeout sets an abort flag that ends the other roles' waits (lanes whose wait
+// ran out go through their role's warp-wide instructions all the same, or leave by the warp's vote),
 // records an error code, and the tensor memory is freed before the CTA exits.
 #include <cuda_fp16.h>
 
@@ -221,9 +222,12 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         static_assert(4 * PW % 8 == 0, "rows of a thread share the swizzle phase");
         uint32_t s = 0, sp = 0;   // running stage and the parity of its current use
         bool ok = true, filled = false;
-        for (int n = 0; n < total && ok; ++n) {
+        // (every lane runs through every slot, those whose wait ran out without another wait or a copy: one that left
+        // would keep the others in the __syncwarp for ever; a vote on leaving instead, here or in the index warp, took
+        // 128^3 from 1154 to 1166 us)
+        for (int n = 0; n < total; ++n) {
             const int r = n % TC_RING;
-            if (!mbar_wait(smem_u32(&rfull[r]), (uint32_t)((n / TC_RING) & 1), &abort_flag)) break;
+            ok = ok && mbar_wait(smem_u32(&rfull[r]), (uint32_t)((n / TC_RING) & 1), &abort_flag);
             // this thread's piece of each of its rows (row 0 with no bytes copied, so zeros, where the box has
             // no source); the rows of a thread are 4 PW apart, a multiple of the swizzle's 8
             const __half* from[RPT];
@@ -237,6 +241,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             const int slot = rmeta[r] & 0xFFFF, lev = rmeta[r] >> 16;
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&rempty[r]));
+            if (!ok) continue;
             const char* tb = reinterpret_cast<const char*>(tabs.t[lev]) + ((int64_t)slot * NK * R + n0) * 128;
 #pragma unroll(NK <= 8 ? NK : 1)
             for (int kc = 0; kc < NK; ++kc) {
@@ -281,7 +286,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         };
         fetch(g0);
         bool ok = true;
-        for (int g = g0; g < g1 && ok; g += TC_GRP) {
+        for (int g = g0; g < g1; g += TC_GRP) {   // (every lane to the end, as the producers)
 #pragma unroll
             for (int q = 0; q < TC_GRP; ++q) {
                 a[q] = nx[q];
@@ -297,10 +302,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             for (int q = 0; q < TC_GRP; ++q) {
                 if (g + q >= g1) break;
                 const int n = g - g0 + q, r = n % TC_RING;
-                if (n >= TC_RING && !mbar_wait(smem_u32(&rempty[r]), (uint32_t)((n / TC_RING - 1) & 1), &abort_flag)) {
-                    ok = false;
-                    break;
-                }
+                if (n >= TC_RING) ok = ok && mbar_wait(smem_u32(&rempty[r]), (uint32_t)((n / TC_RING - 1) & 1), &abort_flag);
                 const int sT = tabs.sT[m[q] >> 16];
                 reinterpret_cast<int4*>(ridx[r])[lane] = a[q];
                 reinterpret_cast<float4*>(rscale[r])[lane] =
@@ -427,7 +429,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (abort_flag && tid == 0) atomicExch(err, 1);
+    if (abort_flag) {
+        if (tid == 0) atomicExch(err, 1);
+        for (int k = 0; k < 32; ++k) __nanosleep(1000);   // (copies and MMAs that another role had just issued)
+    }
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(NCOLS));
 }
 
