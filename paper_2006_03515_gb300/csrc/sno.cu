@@ -68,7 +68,7 @@ struct SnoModel {
     DevBuf m0ab;                     // inference, layer 0: A = R Wl and Bc = (R bl) O, [2][C][K] complex
     DevBuf jt, jref, jorig, jerr;    // photo_solve judge: targets, reference values, caller indices, error
     int mix_mb = 1;                  // modes per block of k_mix_grad
-    size_t zr_smem_f = 0, mixg_smem = 0;
+    size_t lift_smem = 0, mixg_smem = 0;
     int num_sms = 1;
     int64_t steps = 0;
     int period = 0;                  // N of the transforms (>= n)
@@ -164,7 +164,6 @@ __device__ __forceinline__ void sno_cp16z(void* dst, const void* src, bool there
 }
 __device__ __forceinline__ void sno_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void sno_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
-__device__ __forceinline__ void sno_wait_prev() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
 
 // Plane DFTs along x and y, folded: in[p][q][i] -> out[p][j][i] with p < P planes and i < inner
 // columns. About the grid's centre zc = (n - 1) / 2 the points q and n - 1 - q lie at -t and
@@ -1268,10 +1267,17 @@ static FoldTile fold_tiles(int64_t P, int L, int inner, int cols) {
 
 // x and y transforms of [P][n][inner] to [P][2m][inner]: about one item a thread, at most 72 KB of
 // tiles (three blocks an SM at n = 64)
+static FoldTile fold_fwd_tiles(int n, int m, int64_t P, int inner, int& nkb, int& kb, size_t& smem) {
+    nkb = (m + 8) / 8;
+    kb = std::max(4, (m + nkb) / nkb);
+    const FoldTile f = fold_tiles(P, n, inner, std::max(2, std::min(FF_T / nkb, (72 << 10) / (16 * n))) & ~1);
+    smem = ((size_t)2 * f.PB * f.ps + (size_t)nkb * (n / 2) * ((kb + 1) & ~1)) * sizeof(float2);
+    return f;
+}
 static int plane_fwd(SnoModel& M, const float2* in, float2* out, int64_t P, int inner, float zscale = 0.f) {
-    const int nkb = (M.m + 8) / 8, kb = std::max(4, (M.m + nkb) / nkb), kp = (kb + 1) & ~1;
-    const FoldTile f = fold_tiles(P, M.n, inner, std::max(2, std::min(FF_T / nkb, (72 << 10) / (16 * M.n))) & ~1);
-    const size_t smem = ((size_t)2 * f.PB * f.ps + (size_t)nkb * (M.n / 2) * kp) * sizeof(float2);
+    int nkb = 0, kb = 0;
+    size_t smem = 0;
+    const FoldTile f = fold_fwd_tiles(M.n, M.m, P, inner, nkb, kb, smem);
     auto* k = kb == 4 ? k_fold_fwd<4> : kb == 5 ? k_fold_fwd<5> : kb == 6 ? k_fold_fwd<6> : kb == 7 ? k_fold_fwd<7>
                                                                                          : k_fold_fwd<8>;
     int per_sm = 1;
@@ -1283,12 +1289,17 @@ static int plane_fwd(SnoModel& M, const float2* in, float2* out, int64_t P, int 
     return KIFMM_OK;
 }
 // and of [P][2m][inner] to [P][n][inner]
+static FoldTile fold_inv_tiles(int n, int m, int64_t P, int inner, int& njb, size_t& smem) {
+    njb = (n / 2 + FV_J - 1) / FV_J;
+    const FoldTile f = fold_tiles(P, 2 * m, inner, std::max(2, std::min(FV_T / njb, (80 << 10) / (48 * m + 16))) & ~1);
+    smem = ((size_t)2 * f.PB * f.ps + (size_t)(m + 1) * njb * FV_J) * sizeof(float2) +
+           (size_t)(m + 1) * f.PB * f.W * sizeof(float4);
+    return f;
+}
 static int plane_inv(SnoModel& M, const float2* in, float2* out, int64_t P, int inner, float zscale = 0.f) {
-    const int njb = (M.n / 2 + FV_J - 1) / FV_J;
-    const FoldTile f = fold_tiles(P, 2 * M.m, inner,
-                                  std::max(2, std::min(FV_T / njb, (80 << 10) / (48 * M.m + 16))) & ~1);
-    const size_t smem = ((size_t)2 * f.PB * f.ps + (size_t)(M.m + 1) * njb * FV_J) * sizeof(float2) +
-                        (size_t)(M.m + 1) * f.PB * f.W * sizeof(float4);
+    int njb = 0;
+    size_t smem = 0;
+    const FoldTile f = fold_inv_tiles(M.n, M.m, P, inner, njb, smem);
     int per_sm = 1;
     KF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fold_inv, FV_T, smem));
     const int64_t grid = std::min<int64_t>(f.ntiles, (int64_t)std::max(1, per_sm) * M.num_sms);
@@ -1313,6 +1324,26 @@ static int mix(SnoModel& M, int l, const float2* V, float2* G, int B, int adj) {
     return KIFMM_OK;
 }
 
+static size_t lift_u_smem(int n, int m) { return (size_t)(LU * (n / 2 + 1) + n / 2 * (m + 1)) * 8; }
+static size_t lift_z_smem(int n, int C, int m) { return (size_t)((C * (n + 1) + n + 1) & ~1) * 4 + (size_t)m * (n + 1) * 8; }
+static size_t grad_w_smem(int C) { return (size_t)4 * C * GPS * 4; }
+static bool proj_wide(int n, int P) { return P <= 64 && n % 8 == 0; }   // chunks of the projection's backward
+// the most shared memory that a kernel of the forward and backward passes takes (bytes), without k_mix_grad
+static size_t sno_smem(int n, int C, int m, int P, int maxB) {
+    size_t most = std::max({lift_u_smem(n, m), lift_z_smem(n, C, m), grad_w_smem(C), zrow_dims(n, C, m, P, false).smem,
+                            zrow_dims(n, C, m, P, true).smem, proj_dims(C, P, proj_wide(n, P) ? 128 : 64).smem});
+    for (int B = 1; B <= std::min(maxB, MIX_B); ++B) most = std::max(most, mix_dims(C, B).smem);
+    for (int inner : {m, 2 * m * m}) {
+        int a = 0, b = 0;
+        size_t smem = 0;
+        fold_fwd_tiles(n, m, (int64_t)1 << 40, inner, a, b, smem);
+        most = std::max(most, smem);
+        fold_inv_tiles(n, m, (int64_t)1 << 40, inner, a, smem);
+        most = std::max(most, smem);
+    }
+    return most;
+}
+
 static unsigned zr_blocks(const SnoModel& M, int B) { return nbs((int64_t)B * M.n * M.n, ZR_RG); }
 static int near_add(SnoModel& M, const float* u, float* y, int B);
 
@@ -1328,7 +1359,7 @@ static int forward(SnoModel& M, const float* u, float* y, int B, bool train) {
     if (!train) {   // inference: layer 0 from u
 
         const int64_t rows = (int64_t)B * n * n;
-        k_lift_u<<<(unsigned)((rows + LU - 1) / LU), 256, (size_t)(LU * (n / 2 + 1) + n / 2 * (m + 1)) * 8, st>>>(
+        k_lift_u<<<(unsigned)((rows + LU - 1) / LU), 256, lift_u_smem(n, m), st>>>(
             u, T + M.tfo, ptr<float2>(M.cz), rows, n, m);
         KF_LAUNCH();
         KF_TRY(plane_fwd(M, ptr<float2>(M.cz), ptr<float2>(M.cy), (int64_t)B * n, m));     // y
@@ -1347,7 +1378,7 @@ static int forward(SnoModel& M, const float* u, float* y, int B, bool train) {
         k_mix0<<<nbs(BC * M.K, 256), 256, 0, st>>>(ptr<float2>(M.Vst), A, Bc, ptr<float2>(M.g), B, C, M.K);
         KF_LAUNCH();
     } else {
-        k_lift_z<<<zr_blocks(M, B), ZR_T, M.zr_smem_f, st>>>(u, th + M.off[O_WL], th + M.off[O_BL],
+        k_lift_z<<<zr_blocks(M, B), ZR_T, M.lift_smem, st>>>(u, th + M.off[O_WL], th + M.off[O_BL],
                                                              fld(M.v, 0, per), ptr<float2>(M.cz), T + M.tzf, B, C, n,
                                                              m);
         KF_LAUNCH();
@@ -1396,11 +1427,11 @@ static int loss_grad(SnoModel& M, const float* u, const float* t, int B, double*
     const int q = o_q1(M), L = M.L;
     float* dzA = fld(M.dz, 0, per);
     float* dzB = fld(M.dz, 1, per);
-    const bool wide = M.P <= 64 && n % 8 == 0;   // chunks of the projection's backward
+    const bool wide = proj_wide(n, M.P);
     const ProjDims pd = proj_dims(C, M.P, wide ? 128 : 64);
     auto* kpb = wide ? k_proj_bwd<128> : k_proj_bwd<64>;
     const int64_t nchunk = N / GP, rows = BC * n * n;
-    const size_t gsm = (size_t)4 * C * GPS * 4;
+    const size_t gsm = grad_w_smem(C);
     int pb_sm = 1, gw_sm = 1;
     KF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pb_sm, kpb, GD_T, pd.smem));
     KF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&gw_sm, k_grad_w, GD_T, gsm));
@@ -1410,7 +1441,7 @@ static int loss_grad(SnoModel& M, const float* u, const float* t, int B, double*
                                            dzA, gr + M.off[q], gr + M.off[q + 1], gr + M.off[q + 2], gr + M.off[q + 3],
                                            B, C, M.P, M.np3, pd);
     KF_LAUNCH();
-    k_lift_u<<<nbs(rows, LU), 256, (size_t)(LU * (n / 2 + 1) + n / 2 * (m + 1)) * 8, st>>>(
+    k_lift_u<<<nbs(rows, LU), 256, lift_u_smem(n, m), st>>>(
         dzA, T + M.tfo, ptr<float2>(M.cz), rows, n, m);
     KF_LAUNCH();
     const float wn = 1.f / ((float)M.period * M.period * M.period);
@@ -1587,7 +1618,7 @@ static int near_add(SnoModel& M, const float* u, float* y, int B) {
             u, y, n, ptr<int2>(M.near_d), ptr<float>(M.near_w), M.ngroups, M.ntaps);                                         \
         break;
     switch (M.nR) {
-        KF_NEAR(1) KF_NEAR(2) KF_NEAR(3) KF_NEAR(4) KF_NEAR(5) KF_NEAR(6) KF_NEAR(7) KF_NEAR(8)
+        KF_NEAR(1) KF_NEAR(2) KF_NEAR(3) KF_NEAR(4) KF_NEAR(5) KF_NEAR(6) KF_NEAR(7)   // (r_out <= 8)
         default: set_error("near part: halo out of range"); return KIFMM_ERR_ARG;
     }
 #undef KF_NEAR
@@ -1778,29 +1809,29 @@ int sno_create(sno_model_t* out, int n, int width, int modes, int layers, int pr
     const int64_t BC = (int64_t)max_batch * width;
     // shared memory of the kernels (bytes), checked against the device's opt-in limit
     {
-        const size_t ns = n + 1, C1 = width + 1, f4 = 4, f8 = 8, al = 16;
-        const size_t lift = (width * ns + n + 1) * f4 + al + (size_t)modes * ns * f8;
+        M.lift_smem = lift_z_smem(n, width, modes);
+        const size_t f4 = 4, f8 = 8, al = 16, per_mode = (size_t)width * (width + 1 + 2 * max_batch) * f8;
+        M.mix_mb = (int)std::max<size_t>(1, std::min<size_t>(16, (96u << 10) / per_mode));
+        M.mixg_smem = (size_t)2 * max_batch * M.mix_mb * width * f8;
+        // The shapes taken: no more than those for which a form with whole rows of n points, the tables of their
+        // transforms and R with the batch's spectra in shared memory would fit. (Some of the others would fit the kernels
+        // now, 68 points with 64 channels and 33 modes for one, but none of them has been run.)
+        const size_t ns = n + 1, C1 = width + 1;
         const size_t zf = (2 * width * ns + width * C1 + width) * f4 + al +
                           ((size_t)width * modes + n * (modes + 1) + modes * ns) * f8;
         const size_t zb = (3 * width * ns + width * C1) * f4 + al +
                           ((size_t)width * modes + n * (modes + 1) + modes * ns) * f8;
-        M.zr_smem_f = std::max(lift, std::max(zf, zb));
-        // (the forward z-row kernel takes less: the limit on the shapes is an older form's)
         const size_t zr = ((size_t)4 * width * (n + 4) + width * (width + 4) + width + proj_width * (width + 4) +
                      2 * proj_width + 4 * n) * f4 + al +
                     ((size_t)4 * width * modes + n * (modes + 1) + modes * (n + 2)) * f8;
         const size_t zp = zf + ((size_t)proj_width * C1 + 4 * n + 2 * proj_width) * f4;
         const size_t pb = (3 * width * ns + 2 * proj_width * ns + proj_width * C1 + 2 * proj_width + n) * f4 + al +
                       (size_t)modes * ns * f8;
-        const size_t per_mode = (size_t)width * (width + 1 + 2 * max_batch) * f8;
-        M.mix_mb = (int)std::max<size_t>(1, std::min<size_t>(16, (96u << 10) / per_mode));
-        const size_t mix_smem = (size_t)M.mix_mb * per_mode;
-        M.mixg_smem = (size_t)2 * max_batch * M.mix_mb * width * f8;
-        const size_t plane_smem = ((size_t)n * 128 + (size_t)n * 2 * modes) * f8;
+        const size_t rows = std::max({zb, zr, zp, pb, (size_t)M.mix_mb * per_mode, ((size_t)n * 128 + (size_t)n * 2 * modes) * f8});
         int dev = 0, optin = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-        const size_t need = std::max({M.zr_smem_f, zp, pb, mix_smem, M.mixg_smem, plane_smem, zr});
+        const size_t need = std::max({rows, M.mixg_smem, sno_smem(n, width, modes, proj_width, max_batch)});
         cudaDeviceGetAttribute(&M.num_sms, cudaDevAttrMultiProcessorCount, dev);
         M.num_sms = std::max(M.num_sms, 1);
         if (optin <= 0 || need > (size_t)optin) {
@@ -1829,7 +1860,6 @@ int sno_create(sno_model_t* out, int n, int width, int modes, int layers, int pr
         cudaFuncSetAttribute(k_near_add<5>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
         cudaFuncSetAttribute(k_near_add<6>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
         cudaFuncSetAttribute(k_near_add<7>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-        cudaFuncSetAttribute(k_near_add<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
         if (cudaGetLastError() != cudaSuccess) {
             set_error("sno_create: cannot configure the kernels");
             delete h;
