@@ -94,7 +94,10 @@ __global__ void __launch_bounds__(256) k_na_prepare(const double* I, int64_t n, 
 // (a target per lane), every warp of it a contiguous share of the sources, which its lanes load and
 // pass on by shuffles; the shares' sums are added in order, through distributed shared memory. One
 // block of 256 targets each left 4096 points on 16 of the 152 SMs (14.0 ms; with the pairs of
-// pair64.cuh 1.4 ms). CS = 8 below 1216 target groups, so that the last wave is a small part, else 1.
+// pair64.cuh 1.4 ms). CS = 8 below 1216 target groups, eight blocks on each of 152 SMs, else 1: 1000 points
+// 0.12 ms with CS = 8 and 0.36 with 1, 16384 20.6 and 21.6, 30000 68.5 and 69.1, 38912 (1216 groups, one whole wave
+// of single blocks) 115 and 102, 50000 189 and 181, 60000 273 and 256.
+constexpr int NA_CLUSTER_GROUPS = 1216;
 constexpr int NA_T = 256, NA_W = NA_T / 32;
 template <int CS>
 __global__ void __launch_bounds__(NA_T) k_na_direct(const double* __restrict__ pts, const double* I, int n, Pair64 kp,
@@ -216,7 +219,7 @@ extern "C" int kifmm_direct_noalloc(const double* points_dev, int64_t n, double 
     k_na_prepare<<<NA_SIG, 256, 0, st>>>(I_dev, n, h, a, b, self_mode, ws);
     KF_LAUNCH();
     const Pair64 kp = make_pair64(make_kparams(a, b));
-    auto* fn = n <= 32 * 1216 ? launch_na_direct<8> : launch_na_direct<1>;
+    auto* fn = (n + 31) / 32 < NA_CLUSTER_GROUPS ? launch_na_direct<8> : launch_na_direct<1>;
     KF_CUDA(fn(st, points_dev, I_dev, (int)n, kp, C, ws, S_dev));
     return KIFMM_OK;
 }
