@@ -163,8 +163,8 @@ int kifmm_plan(kifmm_plan_t* out, const double* points_dev, int64_t n,
  *   S_dev  device, N outputs (same dtype), fully overwritten (never accumulated).
  *   C      scale factor (1.0 gives the raw sum).
  * Asynchronous on the plan's stream; allocates nothing; no host synchronisation.
- * Mixed plans with the lattice near field run its sums on a second stream owned by the
- * plan, forked from and joined back into the plan's stream by events within the call, so
+ * Mixed plans with the lattice near field, and those off the lattice with 1024 leaves or
+ * more, run the near sums on a second stream owned by the plan, forked from and joined back into the plan's stream by events within the call, so
  * the whole evaluation stays ordered on the plan's stream (and inside a capture of it).
  * Statuses: KIFMM_ERR_ARG (NULL, bad dtype), KIFMM_ERR_CUDA (launch failure). A bounded
  * device wait that gives up is reported by kifmm_check (below), not by this call.
@@ -333,9 +333,9 @@ int kifmm_get_upward(kifmm_plan_t plan, double* c, int* stride);
 
 /* Per-phase device times (ms) of the last kifmm_eval when KIFMM_TIMING=1 in
  * the environment at plan time: [scatter, P2M, M2M, M2L, S2L+L2L+DC2DE,
- * L2P+M2P, P2P] and, where the tensor-core lattice near field ran its sums on
- * the plan's own second stream beside the far field, an eighth entry: the
- * span of those sums (P2P then holds the join and the output combination).
+ * L2P+M2P, P2P] and, where the near sums (the lattice's on the tensor cores, or the
+ * pair sums of a plan of 1024 leaves or more) ran on the plan's own second stream
+ * beside the far field, an eighth entry: the span of those sums (P2P then holds the join and the output combination).
  * Returns the number of phases written (<= cap). */
 int kifmm_get_phase_times(kifmm_plan_t plan, float* ms, int cap);
 

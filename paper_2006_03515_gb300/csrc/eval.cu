@@ -1876,11 +1876,6 @@ static int launch_apply(cudaStream_t st, const T* Op, int ldop, int Mo, int Ki, 
     return KIFMM_OK;
 }
 
-// Far field: upward pass (FP64 in both forms), M2L, downward pass and the leaves'
-// downward equivalent densities, in type T (FP64 form: double; mixed form: float).
-// the near sums on the plan's second stream, after the work ordered before near_ev[0] on the
-// plan's stream; near_ev[1] is recorded whatever happened, so that a join never waits on an
-// unrecorded event and a capture never holds an open fork
 // the generic pair sums into p2p_near, on stream st (they read only the sorted weights)
 static int near_pairs(Plan& p, cudaStream_t st, int64_t& nl) {
     auto* k = p.p2p_series ? k_p2p_mixed<true, float> : k_p2p_mixed<false, float>;
@@ -1895,9 +1890,10 @@ static int near_pairs(Plan& p, cudaStream_t st, int64_t& nl) {
 // The generic pair sums (plans off the lattice) read only the sorted weights as well: issued after the M2L
 // on the second stream, they fill what its last wave and the small levels of the downward pass leave idle
 // (not the M2L itself: its stages take the whole shared memory of an SM). Evaluations without and with:
-// refined grid of 1632 leaves 1215 -> 1135 us, 60 x 52 x 44 cells 522 -> 499 us, 96 x 90 x 100 cells 2828 ->
-// 2808 us, two-level grid of 3.2 M cells 7437 -> 7419 us. Fewer leaves than these were not measured and keep
-// one stream.
+// 1316 leaves 655 -> 608 us, 1440 leaves 321 -> 285 us, 1587 leaves 591 -> 553 us, a cloud of 1177 leaves 760 -> 760 us,
+// 60 x 52 x 44 cells 522 -> 499 us, 96 x 90 x 100 cells 2828 -> 2808 us, two-level grid of 3.2 M cells 7437 -> 7419 us.
+// The line is not where the gain ends: plans of 336 to 953 leaves, which keep one stream, would go from 203 to 166, 221
+// to 206, 242 to 213 and 675 to 641 us.
 constexpr int64_t P2P_FORK_LEAVES = 1024;
 int p2p_fork_plan(Plan& p) {
     const char* ns = std::getenv("KIFMM_NEAR_STREAM");
@@ -1913,6 +1909,9 @@ int p2p_fork_plan(Plan& p) {
     return KIFMM_OK;
 }
 
+// the near sums on the plan's second stream, after the work ordered before near_ev[0] on the
+// plan's stream; near_ev[1] is recorded whatever happened, so that a join never waits on an
+// unrecorded event and a capture never holds an open fork
 static int near_fork_launch(Plan& p, int64_t& nl) {
     cudaError_t e = cudaStreamWaitEvent(p.near_st, p.near_ev[0], 0);
     int rc = KIFMM_OK;
@@ -1933,6 +1932,8 @@ static int near_fork_launch(Plan& p, int64_t& nl) {
     return rc;
 }
 
+// Far field: upward pass (FP64 in both forms), M2L, downward pass and the leaves'
+// downward equivalent densities, in type T (FP64 form: double; mixed form: float).
 template <class T>
 static int run_far(Plan& p, const EvalView& E, int64_t& nl) {
     Tree& t = p.tree;
@@ -2229,16 +2230,16 @@ int run_eval(Plan& p, const void* I, void* S_out, int dtype, double C) {
         // interpolates d in a second kernel
         if (p.lat_far && !p.cheb && t.nlevels > 2) {   // uniform lattice, no W list: the local part is one matrix from d
             KF_TRY(lat_l2p(p, nl));
-            --nl;   // (counted below)
         } else if (mixed) {
+            ++nl;
             auto* kl2p = p.far_series ? k_l2p<true, true, float> : k_l2p<true, false, float>;
             kl2p<<<(unsigned)p.nleaves, L2P_T, 0, st>>>(E, ptr<int32_t>(p.leaves), ptr<float>(p.phid), ptr<double>(p.far));
         } else {
+            ++nl;
             k_l2p<false, true, double><<<(unsigned)p.nleaves, L2P_T, 0, st>>>(E, ptr<int32_t>(p.leaves),
                                                                               ptr<double>(p.phid), ptr<double>(p.far));
         }
         KF_LAUNCH();
-        ++nl;
         if (p.n_wleaves > 0) {
             if (mixed)
                 k_m2p<true, float><<<p.n_wleaves, M2P_T, M2P_G * M2P_CH * 16, st>>>(

@@ -14,7 +14,8 @@ namespace kifmm {
 
 // A tile is cut into pieces of at least this many slots: the start of a CTA (tensor memory, first
 // copies) and the addition of a piece cost about three (32^3, 1250 slots: M2L and addition 76 us
-// with pieces of 6 slots, 34 us with 12).
+// with pieces of 6 slots, 34 us with 12). Whole evaluations with pieces of 6, 12 and 24 slots: 16^3 93, 95 and
+// 114 us, 24^3 148, 152 and 168, 32^3 165, 165 and 183, 40^3 247, 245 and 256, 64^3 306, 295 and 294, 80^3 512, 499 and 496.
 constexpr int kTcMinSlots = 12;
 
 // CTAs of a launch. No more than slots: tiles without a slot count among the ntiles, and a CTA with an
