@@ -44,19 +44,19 @@ METRIC = "S_ph points/s at rel-L2<=1e-6 (FP64 vs mixed KIFMM)"
 # the far-field structure of the 128^3 workload (same M2L launch); the 64^3 capture has its per-leaf
 # shape, and the pair kernel's traffic is compulsory and scales with the point count (x 8 for 128^3).
 PROFILED_TRAFFIC = {
-    "M2L": {"bytes": 165.548e6 + 12.911e6, "per_point_scaled": False,
+    "M2L": {"bytes": 192.552e6 + 19.491e6, "per_point_scaled": False,
             "src": {"paper_2006_03515_gb300/csrc/m2l_tc.cu":
-                    "b8ad63f18f5197f235580d11661f1bafca743abe240f207bc031e4042d8595d5"},
+                    "5c1a6b58789a9b196d4913ed67d894fb2410f656b972acdc24b9178f1b43c8b1"},
             "profile": "profiles/k_m2l_tc_uniform96.md"},
-    "P2P": {"bytes": 14.20e6, "per_point_scaled": True, "n_profiled": 64 ** 3,
+    "P2P": {"bytes": 6.865e6, "per_point_scaled": True, "n_profiled": 64 ** 3,
             "src": {"paper_2006_03515_gb300/csrc/eval.cu":
-                    "27add4c5c6f89bc5081df57c5cc3f95224a7882530864fae517b59636790b1c6"},
+                    "7c4e179a2f6c948236fe729097cf2248e4a7a82b48de614b65a2d29b17ce8ad2"},
             "profile": "profiles/k_p2p_mixed_uniform64.md"},
-    "NEAR": {"bytes": 3.958e6, "per_point_scaled": True, "n_profiled": 64 ** 3,
+    "NEAR": {"bytes": 2.015e6, "per_point_scaled": True, "n_profiled": 64 ** 3,
              "src": {"paper_2006_03515_gb300/csrc/m2l_tc.cu":
-                     "b8ad63f18f5197f235580d11661f1bafca743abe240f207bc031e4042d8595d5",
+                     "5c1a6b58789a9b196d4913ed67d894fb2410f656b972acdc24b9178f1b43c8b1",
                      "paper_2006_03515_gb300/csrc/near_tc.cu":
-                     "46fa6d5f4f4f0e56deeea2645bf8112cb643b02e5a7550efca2993006487a7eb"},
+                     "279f6513caa759be19b6f634e7385b91d9de8ea7a2ea040731bd14276922337d"},
              "profile": "profiles/k_m2l_tc_near_uniform64.md"},
 }
 
